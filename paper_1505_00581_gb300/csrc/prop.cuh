@@ -16,12 +16,13 @@ struct PropLayout {
     int64_t o_W1 = 0, o_b1 = 0, o_W2 = 0, o_b2 = 0, o_w3 = 0, o_b3 = 0, n = 0, n_logical = 0;
 };
 
-// Per-batch activations and scratch of the training kernels.
+// Scratch of the training and forward passes, sized for batches of up to cap rows.
 struct PropTrain {
     void *buf = nullptr;
     int cap = 0;
-    float *z1, *h1, *z2, *h2, *dz2, *dh1, *t_a, *t_b, *spare, *z3, *dz3, *lossv, *loss, *xt, *w2t;
-    int *status;
+    float *part = nullptr;   // per CTA of a pass: its share of the gradient, L.n floats
+    float *loss = nullptr;   // mean loss of the last pass
+    int *status = nullptr;   // 1 once a bounded tensor-core wait gave up
     cudaError_t ensure(const PropLayout &L, int B);
 };
 
@@ -29,12 +30,13 @@ PropLayout prop_layout(int F);
 void prop_pack(const PropLayout &L, const float *logical, std::vector<float> &flat);
 void prop_unpack(const PropLayout &L, const float *flat, float *logical);
 void prop_init(const PropLayout &L, uint64_t seed, std::vector<float> &logical);
+// logits z3 [B] of X [B x d_in] (row stride ldx)
 cudaError_t prop_forward(const PropLayout &L, const float *theta, PropTrain &w, const float *X, int ldx, int B,
-                         cudaStream_t st);
-cudaError_t prop_backward(const PropLayout &L, const float *theta, PropTrain &w, const float *X, int ldx,
-                          const float *y, int B, float *grad, cudaStream_t st);
-cudaError_t prop_adam(const PropLayout &L, float *theta, const float *grad, float *m, float *v, int64_t t, float lr,
-                      cudaStream_t st);
+                         float *logits, cudaStream_t st);
+// gradient of the mean loss on (X, y) into grad (padded layout) and the loss into w.loss; with t > 0 also the t-th
+// Adam step on theta (moments m, v)
+cudaError_t prop_step(const PropLayout &L, float *theta, PropTrain &w, const float *X, int ldx, const float *y, int B,
+                      float *grad, float *m, float *v, int64_t t, float lr, cudaStream_t st);
 
 }  // namespace hgm
 

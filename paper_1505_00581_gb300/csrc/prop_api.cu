@@ -116,9 +116,8 @@ hgm_status hgm_prop_forward(hgm_prop *prop, const float *X, int32_t B, void *str
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = prop->train.ensure(prop->L, B))) return cuerr(e, "workspace");
-    if ((e = prop_forward(prop->L, prop->theta, prop->train, X, prop->L.d_in, B, st))) return cuerr(e, "forward");
-    if ((e = cudaMemcpyAsync(logits, prop->train.z3, sizeof(float) * B, cudaMemcpyDeviceToDevice, st)))
-        return cuerr(e, "copy");
+    if ((e = prop_forward(prop->L, prop->theta, prop->train, X, prop->L.d_in, B, logits, st)))
+        return cuerr(e, "forward");
     return check_status(prop, st);
 }
 
@@ -131,8 +130,8 @@ hgm_status hgm_prop_gradients(hgm_prop *prop, const float *X, const float *y, in
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = prop->train.ensure(prop->L, B))) return cuerr(e, "workspace");
-    if ((e = prop_forward(prop->L, prop->theta, prop->train, X, prop->L.d_in, B, st))) return cuerr(e, "forward");
-    if ((e = prop_backward(prop->L, prop->theta, prop->train, X, prop->L.d_in, y, B, prop->grad, st)))
+    if ((e = prop_step(prop->L, prop->theta, prop->train, X, prop->L.d_in, y, B, prop->grad, prop->m, prop->v, 0, 0.0f,
+                       st)))
         return cuerr(e, "backward");
     hgm_status rc = check_status(prop, st);
     if (rc) return rc;
@@ -154,11 +153,10 @@ hgm_status hgm_prop_train_step(hgm_prop *prop, const float *X, const float *y, i
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = prop->train.ensure(prop->L, B))) return cuerr(e, "workspace");
-    if ((e = prop_forward(prop->L, prop->theta, prop->train, X, prop->L.d_in, B, st))) return cuerr(e, "forward");
-    if ((e = prop_backward(prop->L, prop->theta, prop->train, X, prop->L.d_in, y, B, prop->grad, st)))
-        return cuerr(e, "backward");
+    if ((e = prop_step(prop->L, prop->theta, prop->train, X, prop->L.d_in, y, B, prop->grad, prop->m, prop->v,
+                       prop->step + 1, lr, st)))
+        return cuerr(e, "training step");
     prop->step += 1;
-    if ((e = prop_adam(prop->L, prop->theta, prop->grad, prop->m, prop->v, prop->step, lr, st))) return cuerr(e, "adam");
     if (loss) {
         if ((e = cudaMemcpyAsync(loss, prop->train.loss, sizeof(float), is_dev(loss) ? cudaMemcpyDeviceToDevice
                                                                                           : cudaMemcpyDeviceToHost, st)))

@@ -47,6 +47,14 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
          | ((uint32_t)(M >> 4) << 24);       // M / 16
 }
 
+// The same with either operand MN-major: its rows in memory are the K index and 16-byte chunks run along M (or
+// N), so an operand stored for one product serves another as its transpose. A core matrix is then 8 K x 8 MN;
+// LBO is the byte stride of core matrices along K, SBO along MN (as for K-major operands).
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn, bool b_mn)
+{
+    return idesc_bf16_f32(M, N) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u);
+}
+
 // Byte offset of element (row, k) of a K-major operand in the canonical layout.
 __host__ __device__ __forceinline__ uint32_t kmajor_offset(int row, int k, uint32_t lbo, uint32_t sbo)
 {
