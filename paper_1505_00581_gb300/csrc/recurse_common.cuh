@@ -11,10 +11,13 @@
 
 namespace hgm {
 
+// Approximate square root of a squared angle difference. Flushing subnormal inputs (angle differences below
+// 1.1e-19) saves the compiler's rescaling around the instruction, three more per triple; such a difference is
+// far below an ulp of any angle it is added to.
 __device__ __forceinline__ float sqrt_fast(float x)
 {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 
