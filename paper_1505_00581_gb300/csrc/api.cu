@@ -1647,8 +1647,8 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
     const int T = params->T;
     // band tables per scene (host, from the minnode table): lo(b), cs(b)
     std::vector<int64_t> lo_off((size_t)ns), cs_off((size_t)ns), cell_off((size_t)ns), cells((size_t)ns);
-    std::vector<int32_t> lo_all;
-    std::vector<int64_t> cs_all;
+    std::vector<int32_t> lo_all, flo_all, fhi_all;
+    std::vector<int64_t> cs_all, fr_all;
     int64_t total_cells = 0, max_cells = 0;
     for (int s = 0; s < ns; ++s) {
         const hgm_scene *sc = scenes[s];
@@ -1656,7 +1656,7 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
         const int S = sc->d.S, nf = sc->d.n_frames;
         lo_off[(size_t)s] = (int64_t)lo_all.size();
         cs_off[(size_t)s] = (int64_t)cs_all.size();
-        int64_t c = 0;
+        int64_t c = 0, fr = 0;
         for (int f = 0; f < nf; ++f) {
             const int lo = T > 0 ? fs[(size_t)std::max(0, f - T + 1)] : 0;
             const int reach = (T > 0 ? fs[(size_t)std::min(nf, f + T)] : S) - fs[(size_t)f];
@@ -1665,11 +1665,16 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
                             reach, f);
             for (int b = fs[(size_t)f]; b < fs[(size_t)f + 1]; ++b) {
                 lo_all.push_back(lo);
+                flo_all.push_back(fs[(size_t)f]);
+                fhi_all.push_back(fs[(size_t)f] + reach);
                 cs_all.push_back(c);
+                fr_all.push_back(fr);
                 c += fs[(size_t)f + 1] - lo;
+                fr += block_row(reach);
             }
         }
         cs_all.push_back(c);
+        fr_all.push_back(fr);
         cells[(size_t)s] = c;
         cell_off[(size_t)s] = total_cells;
         total_cells += c;
@@ -1693,22 +1698,36 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
     }
     const int R = bb.R;
     const int Fp = models[0]->d.F;
+    std::vector<BlockBand> bands((size_t)ns);
+    int max_M = 0;
+    for (int m = 0; m < nm; ++m) max_M = std::max(max_M, models[m]->d.M);
+    for (int s = 0; s < ns; ++s)
+        bands[(size_t)s] = BlockBand{scenes[s]->d.S, scenes[s]->d.n_frames, lo_all.data() + lo_off[(size_t)s],
+                                     flo_all.data() + lo_off[(size_t)s], fhi_all.data() + lo_off[(size_t)s],
+                                     cs_all.data() + cs_off[(size_t)s],
+                                     fr_all.data() + cs_off[(size_t)s]};
+    const BlockPlan plan = block_plan(bands.data(), ns, (int)units.size(), max_M, T);
+    std::vector<int32_t> fr32(plan.shared ? fr_all.size() : 0);   // rows of shared scenes hold < 2^31 entries
+    for (size_t k = 0; k < fr32.size(); ++k) fr32[k] = (int32_t)fr_all[k];
     int64_t S_total = 0;
     std::vector<int64_t> u_off((size_t)ns);
     for (int s = 0; s < ns; ++s) {
         u_off[(size_t)s] = S_total * R;
         S_total += scenes[s]->d.S;
     }
-    // one upload: [lo | cs | units | scene records | band records], each part 256-byte aligned
+    // one upload: [lo | cs | units | scene records | band records | fr], each part 256-byte aligned
     auto al256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
     const size_t o_cs = al256(lo_all.size() * sizeof(int32_t));
     const size_t o_units = o_cs + al256(cs_all.size() * sizeof(int64_t));
     const size_t o_srec = o_units + al256(units.size() * sizeof(BlockUnit));
     const size_t o_geo = o_srec + al256((size_t)ns * sizeof(SceneRec));
-    const size_t tab_bytes = o_geo + al256((size_t)ns * sizeof(BlockGeo));
+    const size_t o_fr = o_geo + al256((size_t)ns * sizeof(BlockGeo));
+    const size_t tab_bytes = o_fr + al256(fr32.size() * sizeof(int32_t));
     CK(bb.tab.ensure(tab_bytes), "workspace (block)");
-    CK(bb.cellb.ensure((size_t)std::max<int64_t>(total_cells, 1) * sizeof(int32_t)), "workspace (block)");
-    CK(bb.dir.ensure((size_t)std::max<int64_t>(total_cells, 1) * 2 * sizeof(float)), "workspace (block)");
+    if (!plan.shared) {
+        CK(bb.cellb.ensure((size_t)std::max<int64_t>(total_cells, 1) * sizeof(int32_t)), "workspace (block)");
+        CK(bb.dir.ensure((size_t)std::max<int64_t>(total_cells, 1) * 2 * sizeof(float)), "workspace (block)");
+    }
     CK(bb.U.ensure((size_t)std::max<int64_t>(S_total * R, 1) * sizeof(float)), "workspace (block)");
     CK(bb.beta.ensure(beta_bytes), "workspace (block)");
     char *dtab = bb.tab.as<char>();
@@ -1719,9 +1738,18 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
     float *dirf_all = bb.dir.as<float>(), *dirb_all = dirf_all + total_cells;
     for (int s = 0; s < ns; ++s) {
         const hgm_scene *sc = scenes[s];
-        geos[(size_t)s] = BlockGeo{d_lo + lo_off[(size_t)s], d_cs + cs_off[(size_t)s],
-                                   bb.cellb.as<int32_t>() + cell_off[(size_t)s], dirf_all + cell_off[(size_t)s],
-                                   dirb_all + cell_off[(size_t)s], cells[(size_t)s]};
+        BlockGeo &g = geos[(size_t)s];
+        g = BlockGeo{d_lo + lo_off[(size_t)s], d_cs + cs_off[(size_t)s], nullptr, nullptr, nullptr, nullptr,
+                     cells[(size_t)s], {}, {}};
+        if (plan.shared) {
+            g.fr = reinterpret_cast<const int32_t *>(dtab + o_fr) + cs_off[(size_t)s];
+            block_split(bands[(size_t)s], plan.csize, g.split);
+            for (int r = 0; r <= plan.csize; ++r) g.split_fr[r] = (int32_t)bands[(size_t)s].fr[g.split[r]];
+        } else {
+            g.cellb = bb.cellb.as<int32_t>() + cell_off[(size_t)s];
+            g.dirf = dirf_all + cell_off[(size_t)s];
+            g.dirb = dirb_all + cell_off[(size_t)s];
+        }
         srec[(size_t)s] = SceneRec{sc->d.xy, sc->d.t, sc->d.frame_start, sc->d.perm, bb.U.as<float>() + u_off[(size_t)s],
                                    (int64_t)sc->d.S, sc->d.S, sc->d.n_frames, sc->d.f, nullptr, 0};
     }
@@ -1747,14 +1775,16 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
     std::memcpy(h + o_units, units.data(), units.size() * sizeof(BlockUnit));
     std::memcpy(h + o_srec, srec.data(), srec.size() * sizeof(SceneRec));
     std::memcpy(h + o_geo, geos.data(), geos.size() * sizeof(BlockGeo));
+    if (!fr32.empty()) std::memcpy(h + o_fr, fr32.data(), fr32.size() * sizeof(int32_t));
     CK(cudaMemcpyAsync(dtab, h, tab_bytes, cudaMemcpyHostToDevice, st), "upload block tables");
     if (bb.own_pinned) CK(cudaEventRecord(bb.upload_done, st), "event");
     for (int s = 0; s < ns; ++s) {
         const hgm_scene *sc = scenes[s];
         const BlockGeo &g = geos[(size_t)s];
-        CK(launch_block_geo(sc->d.xy, sc->d.S, g.lo, g.cs, g.cells, const_cast<int32_t *>(g.cellb),
-                            const_cast<float *>(g.dirf), const_cast<float *>(g.dirb), st),
-           "block geometry");
+        if (!plan.shared)
+            CK(launch_block_geo(sc->d.xy, sc->d.S, g.lo, g.cs, g.cells, const_cast<int32_t *>(g.cellb),
+                                const_cast<float *>(g.dirf), const_cast<float *>(g.dirb), st),
+               "block geometry");
         if (sc->d.S > 0)
             CK(launch_unary(bb.model.as<float>(), R, sc->d.f, sc->d.S, Fp, params->lambda1,
                             const_cast<float *>(srec[(size_t)s].U), sc->d.S, st),
@@ -1777,9 +1807,7 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
     p.F = Fp;
     float *scratch = nullptr;
     int grid_global = 0;
-    static int64_t smem_cells = -1;
-    if (smem_cells < 0) smem_cells = block_smem_cells();
-    if (max_cells > smem_cells) {
+    if (!plan.shared) {
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev), "device");
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");
@@ -1789,7 +1817,7 @@ hgm_status run_block(BlockBufs &bb, const hgm_model *const *models, int nm, cons
     }
     CK(launch_block_recurse(reinterpret_cast<const BlockUnit *>(rec), (int)units.size(), bb.mrec.as<ModelRec>(),
                             reinterpret_cast<const SceneRec *>(rec + b_units),
-                            reinterpret_cast<const BlockGeo *>(rec + b_units + b_s), p, max_cells,
+                            reinterpret_cast<const BlockGeo *>(rec + b_units + b_s), p, plan, max_cells,
                             bb.beta.as<uint16_t>(), scratch, grid_global, de, da, st),
        "block recursion kernel");
     if (energy && !e_dev)
@@ -1873,7 +1901,7 @@ hgm_status stream_reserve(hgm_stream *s, int64_t P, cudaStream_t st)
     BlockBufs &bb = s->bb;
     auto al256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
     const size_t tab = al256((size_t)P * 4) + al256((size_t)(P + 1) * 8) + al256((size_t)nm * sizeof(BlockUnit)) +
-                       al256(sizeof(SceneRec)) + al256(sizeof(BlockGeo));
+                       al256(sizeof(SceneRec)) + al256(sizeof(BlockGeo)) + al256((size_t)(P + 1) * 4);
     const int64_t cells = std::max<int64_t>(P * P, 1);
     CK(bb.tab.ensure(tab), "stream buffers");
     CK(cudaMallocHost(&bb.pinned, tab), "pinned staging");
@@ -1884,7 +1912,7 @@ hgm_status stream_reserve(hgm_stream *s, int64_t P, cudaStream_t st)
     CK(bb.beta.ensure((size_t)std::max<int64_t>(Rm2 * cells, 1) * sizeof(uint16_t)), "stream buffers");
     CK(bb.oe.ensure((size_t)nm * sizeof(float)), "stream buffers");
     CK(bb.oa.ensure((size_t)std::max<int64_t>(R, 1) * sizeof(int32_t)), "stream buffers");
-    if (cells > block_smem_cells()) {
+    if (!block_always_shared(P, B, s->params.T)) {
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev), "device");
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");

@@ -185,14 +185,36 @@ cudaError_t preload_backtrack();
 
 // Profiling hooks (api.cu).
 // k_block.cu: the whole-block problem (every scene point a candidate, no offsets).
+constexpr int kMaxCluster = 8;   // CTAs of a cluster (the portable limit)
 struct BlockGeo {            // band tables of one scene (see k_block.cu)
     const int32_t *lo;       // [S] first point of b's band
     const int64_t *cs;       // [S+1] first cell of b's band
-    const int32_t *cellb;    // [cells] owner b of each cell
-    const float *dirf;       // [cells] theta(b->c)
-    const float *dirb;       // [cells] theta(c->b)
+    const int32_t *fr;       // [S+1] first entry of b's forward row (shared-memory form)
+    const int32_t *cellb;    // [cells] owner b of each cell (global form)
+    const float *dirf;       // [cells] theta(b->c) (global form)
+    const float *dirb;       // [cells] theta(c->b) (global form)
     int64_t cells;
+    int32_t split[kMaxCluster + 1];      // points of a cluster's CTAs: [split[r], split[r + 1])
+    int32_t split_fr[kMaxCluster + 1];   // fr of those points
 };
+// Entries of a forward row of n points: padded to an even length with at least one entry to spare.
+__host__ __device__ inline int block_row(int n) { return (n + 2) & ~1; }
+// The band of one scene on the host: lo and cs as above, the row's points [flo(b), fhi(b)), fr as above (64 bits).
+struct BlockBand {
+    int S, n_frames;
+    const int32_t *lo, *flo, *fhi;
+    const int64_t *cs, *fr;
+};
+// How a whole-block call runs. shared: tables in shared memory, csize CTAs per pair; else global scratch.
+struct BlockPlan {
+    bool shared = false;
+    int csize = 1, threads = 0, clusters = 0;
+    int rows = 0, trows = 0, cells = 0, pts = 0, beta = 0;   // BlockShape of k_block.cu
+};
+BlockPlan block_plan(const BlockBand *bands, int n_scenes, int n_units, int max_M, int T);
+void block_split(const BlockBand &bd, int csize, int32_t *split);   // csize + 1 entries
+// true if every block of up to `points` points over n_frames frames runs in one CTA's shared memory
+bool block_always_shared(int64_t points, int n_frames, int T);
 struct BlockUnit {
     int32_t model, scene;
     int64_t beta;            // first argmin entry (uint16) of this unit: (M-2) x cells
@@ -200,12 +222,10 @@ struct BlockUnit {
 };
 cudaError_t launch_block_geo(const float2 *xy, int S, const int32_t *lo, const int64_t *cs, int64_t cells,
                              int32_t *cellb, float *dirf, float *dirb, cudaStream_t st);
-int64_t block_smem_cells();   // largest band table (cells) whose two copies fit one CTA's shared memory
-// scratch == nullptr: tables in shared memory (max_cells <= block_smem_cells()); else per-CTA global scratch
-// of 2 x max_cells floats for grid_global CTAs.
+// global form: scratch of grid_global x 2 x max_cells floats
 cudaError_t launch_block_recurse(const BlockUnit *units, int n_units, const ModelRec *models, const SceneRec *scenes,
-                                 const BlockGeo *geos, Params p, int64_t max_cells, uint16_t *beta, float *scratch,
-                                 int grid_global, float *energy, int32_t *assign, cudaStream_t st);
+                                 const BlockGeo *geos, Params p, const BlockPlan &pl, int64_t max_cells, uint16_t *beta,
+                                 float *scratch, int grid_global, float *energy, int32_t *assign, cudaStream_t st);
 
 // k_dummy.cu: the recursion with the dummy assignment eps (fused backtrack; per-CTA argmin scratch).
 // evaluated != NULL runs the accounting variant, which adds its evaluated triples to *evaluated.
