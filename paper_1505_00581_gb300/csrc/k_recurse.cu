@@ -37,19 +37,17 @@
 // triple loop, in increasing slot order with a strict '<', so the lowest slot
 // still wins exact ties -- the result is bit-identical to the full minimisation.
 //
-// Work split per step (three CTA barriers): phase 1, NP threads per b (adjacent
-// lanes, interleaved a) build the kept lists with pairwise shuffles only, while
-// the other warps compute the theta(a->c) table; then every thread takes part in
-// ordering the b by decreasing kept count and laying out the tile table; phase
-// 3, tiles of one b and CT consecutive c with
-// t'(c) <= t'(b) are flattened across the CTA's threads in that order (similar
-// loop lengths within a warp), each thread looping over the kept a of its b.
-// The per-step model constants come from a table built at model creation, and
-// the list C of the next step is fetched from global memory during phase 2 and
-// stored in the buffer of the list A, which phase 3 no longer reads, so no step
-// waits on a global load. Argmin bytes are written for the tiled cells only, a
-// tile's four at once: the cells past b's time prefix are never on a chain, so
-// the backtrack never reads them.
+// Work split per step (three CTA barriers): phase 1, NT / KM threads per b, each with a run of row b's base in
+// registers, find the row's two smallest, its threshold and its kept list with shuffles among neighbours only (the
+// bisections of list C go to different lanes); the same threads then fill the theta(a->c) table; then every thread
+// takes part in ordering the b by decreasing kept count and laying out the tile table; phase 3, tiles of one b and
+// CT consecutive c with t'(c) <= t'(b) are flattened across the CTA's threads in that order (similar loop lengths
+// within a warp), each thread looping over the kept a of its b. A cell's alpha_i(b,c) is written as the next step's
+// base: with a = b and b = c it is U(b) + lambda2 Delta(b,c) + alpha_i(b,c), the same Delta as in alpha itself.
+// The per-step model constants come from a table built at model creation, and the list C of the next step is
+// fetched from global memory during phase 1 and stored in the buffer of the list A, which phase 3 no longer reads,
+// so no step waits on a global load. Argmin bytes are written for the tiled cells only, a tile's four at once: the
+// cells past b's time prefix are never on a chain, so the backtrack never reads them.
 #include "backtrack.cuh"
 #include "recurse_common.cuh"
 
@@ -58,21 +56,6 @@ namespace {
 
 constexpr float kInf = __builtin_huge_valf();
 constexpr float kGeoMax = 4.45f;   // > pi*sqrt(2) = 4.4429, bound of the FP32 D^g
-
-__device__ __forceinline__ uint32_t lanemask_lt()
-{
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
-
-// Kept entry k of b sits at a per-row rotation of its slot, so that the rows of different b -- whose
-// starts are multiples of 32 banks apart -- spread over the banks when several b are read or written
-// at the same position (phase 1 writes, the triple loop's reads).
-template <int KM>
-__device__ __forceinline__ int fb_at(int b, int k) { return b * KM + ((k + b) & (KM - 1)); }
-template <int KM>
-__device__ __forceinline__ int fs_at(int b, int k) { return b * KM + ((k + 4 * b) & (KM - 1)); }
 
 template <int KM>
 struct alignas(16) List {   // 16-byte aligned arrays: tiles read four consecutive entries at once
@@ -83,27 +66,29 @@ struct alignas(16) List {   // 16-byte aligned arrays: tiles read four consecuti
     int32_t n;
 };
 
-template <int KM, int NT, int NP>
+template <int KM, int NT>
 struct Smem {
-    static constexpr int RS = KM + 4;     // row stride of r (16-byte rows, bank skew)
-    float2 fb[KM * KM];                   // per b: kept (base, p1) in increasing a, at b*KM + k
-    float r[KM * RS];                     // theta(a->c) or +inf, at a*RS + c
-    // row stride of alpha: phase 1 reads row b at a = NP k + h with lanes (b, h); conflict-free when
-    // AS = NP (mod 32) and odd multiples are avoided: 65 for one thread per b, 66 for two
-    static constexpr int AS = KM + NP;
-    float alpha[KM * AS];                 // alpha_{i+1}(a,b) at b*AS + a (then base(a,b)); alpha_i(b,c) at c*AS + b
-    uint8_t fs[KM * KM];                  // slot a of each kept entry, | 0x80 when a lies at b's position
-    uint8_t fn[KM];                       // number of kept a per b
-    uint8_t tile_b[KM * KM / 4];          // b of every tile of the step (tiles of >= 4 cells)
-    uint16_t tbase[KM];                   // first tile of b
-    uint8_t tcount[KM];                   // tiles of b
-    int32_t pw[KM];                       // per b: (sort key << 5) | tile count, key 0 for b without tiles
-    int32_t ntile;                        // tiles of the step
+    // row strides: rows of different b read at the same place fall into different banks (FS, SS); rows of r and
+    // alpha are whole 16-byte groups whose starts are 4 banks apart, and their four words past the KM columns hold
+    // the step's tile table
+    static constexpr int FS = KM + 1, SS = KM + 4, RS = KM + 4, AS = KM + 4;
+    float2 fb[KM * FS];                   // per b: kept (base, p1) in increasing a
+    float r[KM * RS];                     // theta(a->c) or +inf, at a*RS + c | 16 bytes of tile_b per row
+    float alpha[KM * AS];                 // base(a,b) of the coming step at b*AS + a | rank key, tile info of b
+    uint8_t fs[KM * SS];                  // slot a of each kept entry, | 0x80 when a lies at b's position
     List<KM> list[3];
     float4 geo[2];                        // model constants of step i at geo[i & 1]
     float red_v[NT / 32];
     int32_t red_k[NT / 32];
+    int32_t ntile;                        // tiles of the step
     int32_t unit;
+    int32_t coin[2];                      // step i: some kept a lies at its b's position (coin[i & 1])
+
+    // b of tile t (tiles of >= 4 cells); per b: (sort key << 5) | tile count, key 0 for b without tiles; first tile
+    // << 12 | kept count << 5 | tile count
+    __device__ uint8_t &tile_b(int t) { return reinterpret_cast<uint8_t *>(&r[(t >> 4) * RS + KM])[t & 15]; }
+    __device__ int32_t &key(int b) { return reinterpret_cast<int32_t *>(alpha)[b * AS + KM]; }
+    __device__ int32_t &info(int b) { return reinterpret_cast<int32_t *>(alpha)[b * AS + KM + 1]; }
 };
 
 template <int KM>
@@ -141,8 +126,8 @@ __device__ __forceinline__ void argmin_merge(float &v, int &k, float ov, int ok)
 // live in a per-CTA scratch block (beta + blockIdx.x * beta_cta, reused unit
 // after unit), and the CTA backtracks its own unit and writes the energy and
 // the assignment itself.
-template <int KM, int NT, int CT, int NP, int UR, bool kCount, bool kFused>
-__global__ void __launch_bounds__(NT, (KM > 32 ? 3 : 4))
+template <int KM, int NT, int MB, int CT, int UR, bool kCount, bool kFused>
+__global__ void __launch_bounds__(NT, MB)
 recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *__restrict__ models,
                const SceneRec *__restrict__ scenes, Params p, const int32_t *__restrict__ cand_idx,
                const float *__restrict__ cand_u, const int32_t *__restrict__ cand_cnt, uint8_t *__restrict__ beta,
@@ -156,21 +141,23 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
     }
     unsigned long long n_eval = 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem<KM, NT, NP> &sm = *reinterpret_cast<Smem<KM, NT, NP> *>(smem_raw);
-    constexpr int RS = Smem<KM, NT, NP>::RS;
-    constexpr int AS = Smem<KM, NT, NP>::AS;
-    constexpr int AQ = KM / 32;            // slots per lane in warp-wide passes
+    using SM = Smem<KM, NT>;
+    SM &sm = *reinterpret_cast<SM *>(smem_raw);
+    constexpr int RS = SM::RS, AS = SM::AS, FS = SM::FS, SS = SM::SS;
     constexpr int NW = NT / 32;
-    constexpr int P1 = KM * NP;            // threads building the kept lists (NP per b); the rest: theta table
-    constexpr int AH = KM / NP;            // a (and c) slots per list-building thread
-    static_assert(NP == 1 || NP == 2, "one or two threads per b");
-    static_assert(P1 % 32 == 0 && NT - P1 >= KM, "thread split");
+    constexpr int TPB = NT / KM;           // threads per b (and per c): neighbouring lanes
+    constexpr int AH = KM / TPB;           // slots a per thread: a = AH h + 0 .. AH - 1
+    static_assert(TPB == 4 || TPB == 8, "threads per b");
+    const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = p.K;
     const int T = p.T;
     const float lam2 = p.lambda2;
     const float lam23 = p.lambda2 * p.lambda3;
     const float gmax = lam23 * kGeoMax;
+    const int h = tid % TPB, row = tid / TPB;
+    // a thread reads its run of slots from a start of its own, so that a warp's reads hit every bank once
+    const int rot = TPB == 4 ? h : (h & 1) + ((h >> 2) << 1);
 
     for (;;) {
         if (tid == 0) sm.unit = atomicAdd(work_counter, 1);
@@ -189,12 +176,25 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
         const int32_t *ccnt = cand_cnt + un.cand / K;
         uint8_t *ubeta = kFused ? beta + (int64_t)blockIdx.x * beta_cta : beta + un.beta;
 
-        // alpha_{M+1} == 0 (Eq. 11); the three lists and the constants of the first step
-        for (int e = tid; e < KM * AS; e += NT) sm.alpha[e] = 0.0f;
+        // the three lists and the constants of the first step
         for (int q = 1; q <= 3 && q <= M; ++q)
             load_list<KM>(sm.list[(M - q) % 3], sc, cidx + (int64_t)(M - q) * K, cu + (int64_t)(M - q) * K,
                           ccnt[M - q], tid, NT);
-        if (tid == 0 && M >= 3) sm.geo[(M - 1) & 1] = md.geo[M - 1];
+        if (tid == 0 && M >= 3) {
+            sm.geo[(M - 1) & 1] = md.geo[M - 1];
+            sm.coin[0] = sm.coin[1] = 0;
+        }
+        __syncthreads();
+        {   // the first step's base: alpha_{M+1} == 0 (Eq. 11)
+            const List<KM> &LA = sm.list[(M - 1) % 3], &LB = sm.list[(M - 2) % 3];
+            const int dt_ab = __float_as_int(sm.geo[(M - 1) & 1].z);
+            for (int e = tid; e < KM * KM; e += NT) {
+                const int b = e / KM, a = e % KM;
+                // slots past a list hold t = 0x3fffffff, idx = -1, u = inf
+                const bool ok = a < LA.n && b < LB.n && LA.t[a] >= LB.t[b] && LA.idx[a] != LB.idx[b];
+                sm.alpha[b * AS + a] = ok ? base_cost(LA.u[a], lam2, dt_ab, LA.t[a], LB.t[b], 0.0f) : kInf;
+            }
+        }
         __syncthreads();
 
         for (int i = M - 1; i >= 2; --i) {
@@ -206,197 +206,174 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // p2 = p1 + k2 uses theta(a->b) = theta(b->a) + pi, which fails for a and b at the same position
             // (both directions are atan2(0, 0) = 0, reading R1): such entries (flagged in fs) take k2c
             const float k2c = wrap_pi(__fsub_rn(k2, kPi));
-            const int dt_ab = __float_as_int(g.z), dt_bc = __float_as_int(g.w);
+            const int dt_bc = __float_as_int(g.w);
             const int na = LA.n, nb = LB.n, nc = LC.n;
 
-            // list C of the next step (chain index i-3) is fetched by the theta-table threads
-            const int pfi = tid - P1;
-            const bool pf = i >= 3 && pfi >= 0 && pfi < K;
+            // list C of the next step (chain index i-3) is fetched by the first threads
+            const bool pf = i >= 3 && tid < K;
             int pf_n = 0, pf_j = -1;
             float pf_u = kInf;
             float2 pf_xy = make_float2(0.f, 0.f);
             int pf_t = 0x3fffffff;
-            bool pf_ok = false;
+            if (pf) {
+                pf_n = ccnt[i - 3];
+                pf_j = cidx[(int64_t)(i - 3) * K + tid];
+                pf_u = cu[(int64_t)(i - 3) * K + tid];
+            }
+            if (tid == NT - 1 && i >= 3) sm.geo[(i - 1) & 1] = md.geo[i - 1];
 
-            if (tid < P1) {
-                // ---- phase 1: the kept a list of b, NP threads per b (lanes h of a pair; a = NP k + h)
-                const int b = tid / NP, h = tid % NP;
+            // ---- phase 1: the kept a list of b = row
+            {
+                const int b = row;
                 const bool inb = b < nb;
                 float2 pb = make_float2(0.f, 0.f);
                 int tb = 0, ib = -1;
                 if (inb) { pb = LB.xy[b]; tb = LB.t[b]; ib = LB.idx[b]; }
-                float *arow = sm.alpha + b * AS;
-                // smallest and second-smallest base (value, slot) over all feasible a
-                float m1 = kInf, m2 = kInf;
-                int s1 = 1 << 20, s2 = 1 << 20;
+                const float *arow = sm.alpha + b * AS + AH * h;
                 // the a with t'(a) >= t'(b) form a suffix of list A (time order): the slots before it are never
-                // feasible with b and are neither evaluated nor read below (k0: first k that can reach it)
-                int k0 = 0;
-                if (inb) {
-                    int lo = 0, hi = na;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (LA.t[mid] < tb) lo = mid + 1;
-                        else hi = mid;
-                    }
-                    k0 = lo / NP;
+                // feasible with b, and the row holds nothing of this step there
+                int lo = 0;
+                for (int hi = inb ? na : 0; lo < hi;) {
+                    const int mid = (lo + hi) >> 1;
+                    if (LA.t[mid] < tb) lo = mid + 1;
+                    else hi = mid;
                 }
-                if (inb) {
-#pragma unroll 4
-                    for (int k = k0; k < AH; ++k) {
-                        const int a = NP * k + h;
-                        // slots past the list hold t = 0x3fffffff, idx = -1, u = inf: never feasible with b
-                        const int ta = LA.t[a];
-                        float bs = kInf;
-                        if (a < na && ta >= tb && LA.idx[a] != ib)
-                            bs = base_cost(LA.u[a], lam2, dt_ab, ta, tb, arow[a]);
-                        arow[a] = bs;   // base(a,b) replaces alpha_{i+1}(a,b): read once, by this thread
-                        if (bs < m1) { m2 = m1; s2 = s1; m1 = bs; s1 = a; }
-                        else if (bs < m2) { m2 = bs; s2 = a; }
-                    }
+                const int j0 = lo - AH * h, j1 = (inb ? na : 0) - AH * h;
+                // smallest and second smallest base over all feasible a
+                float v[AH], m1 = kInf, m2 = kInf;
+#pragma unroll
+                for (int k = 0; k < AH; ++k) {
+                    const int j = (k + rot) & (AH - 1);
+                    const float x = arow[j];
+                    v[k] = j >= j0 && j < j1 ? x : kInf;
+                    m2 = fminf(m2, fmaxf(m1, v[k]));
+                    m1 = fminf(m1, v[k]);
                 }
-                if constexpr (NP == 2) {
-                    // merge the pair's (value, slot) top-2 lists; ties go to the lower slot
-                    const float om1 = __shfl_xor_sync(0xffffffffu, m1, 1), om2 = __shfl_xor_sync(0xffffffffu, m2, 1);
-                    const int os1 = __shfl_xor_sync(0xffffffffu, s1, 1), os2 = __shfl_xor_sync(0xffffffffu, s2, 1);
-                    if (om1 < m1 || (om1 == m1 && os1 < s1)) {
-                        if (m1 < om2 || (m1 == om2 && s1 < os2)) { m2 = m1; s2 = s1; }
-                        else { m2 = om2; s2 = os2; }
-                        m1 = om1; s1 = os1;
-                    } else if (om1 < m2 || (om1 == m2 && os1 < s2)) {
-                        m2 = om1; s2 = os1;
-                    }
+#pragma unroll
+                for (int off = 1; off < TPB; off <<= 1) {
+                    const float o1 = __shfl_xor_sync(full, m1, off), o2 = __shfl_xor_sync(full, m2, off);
+                    m2 = fminf(fmaxf(m1, o1), fminf(m2, o2));
+                    m1 = fminf(m1, o1);
                 }
-                const float bv = m1;
-                // c with t'(c) <= t'(b) form a prefix of C (time order): its length by binary search
-                int ccount = 0;
-                if (inb) {
-                    int lo = 0, hi = nc;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (LC.t[mid] <= tb) lo = mid + 1;
-                        else hi = mid;
+                // lowest slot of a value among the row's (1 << 20: none)
+                auto slot_of_value = [&](float x, int skip) {
+                    int s = 1 << 20;
+#pragma unroll
+                    for (int k = 0; k < AH; ++k) {
+                        const int a = AH * h + ((k + rot) & (AH - 1));
+                        if (v[k] == x && a != skip) s = min(s, a);
                     }
-                    ccount = lo;
+#pragma unroll
+                    for (int off = 1; off < TPB; off <<= 1) s = min(s, __shfl_xor_sync(full, s, off));
+                    return s;
+                };
+                const bool any = m1 < kInf;
+                int s1 = slot_of_value(m1, -1);   // every lane takes part in the exchanges
+                if (!any) s1 = 0;
+                const int tw = LA.t[s1], iw = any ? LA.idx[s1] : -2;
+                // C is in increasing scene index, hence in increasing time: the c with t'(c) <= x form a prefix, and
+                // a point's slot is found by bisection. Four lanes take one search each: c not after b, c too far
+                // from the witness, b's point, the witness's point.
+                auto lower_bound = [&](const int32_t *arr, int x) {
+                    int l = 0, r = nc;
+                    while (l < r) {
+                        const int mid = (l + r) >> 1;
+                        if (arr[mid] < x) l = mid + 1;
+                        else r = mid;
+                    }
+                    return l;
+                };
+                const int base_lane = lane & ~(TPB - 1);
+                int ccount, nT, pbs, pw;
+                {
+                    const int q = h & 3;
+                    const int32_t *arr = q < 2 ? LC.t : LC.idx;
+                    const int x = q == 0 ? tb + 1 : q == 1 ? (T > 0 ? tw - T + 1 : INT32_MIN) : q == 2 ? ib : iw;
+                    int f = lower_bound(arr, x);
+                    if (q >= 2 && !(f < nc && arr[f] == x)) f = KM;
+                    ccount = __shfl_sync(full, f, base_lane);
+                    if (!inb) ccount = 0;
+                    nT = min(__shfl_sync(full, f, base_lane + 1), ccount);
+                    pbs = __shfl_sync(full, f, base_lane + 2);
+                    pw = __shfl_sync(full, f, base_lane + 3);
                 }
-                const bool live = inb && bv < kInf && ccount > 0;
-                // cells (b,c) where the witness s1 is infeasible: their best base is the second smallest over
-                // the a feasible with c -- exactly m2 when the runner-up s2 is feasible with c; otherwise
-                // (rare) every a is kept
-                bool anybad = false, loose = false;
-                if (live) {
-                    // C is in increasing scene index, hence in increasing time: the c with t'(c) <= x form a
-                    // prefix, and a point's slot in C is found by bisection. The cells of b's own point are
-                    // infeasible and never count; the witness and the runner-up are feasible with b, so their
-                    // points differ from b's.
-                    const int tw = LA.t[s1], iw = LA.idx[s1];
+                const bool live = any && ccount > 0;
+                // cells (b,c) where the witness s1 is infeasible (the cells of b's own point never count; witness and
+                // runner-up are feasible with b, so their points differ from b's): their best base is the second
+                // smallest over the a feasible with c -- exactly m2 when the runner-up s2 is feasible with c;
+                // otherwise (rare) every a is kept
+                const bool anybad = live && (nT - (pbs < nT ? 1 : 0) > 0 || pw < ccount);
+                bool loose = false;
+                if (__any_sync(full, anybad)) {
                     const bool has2 = m2 < kInf;
+                    const int s2 = slot_of_value(m2, s1);
                     const int t2 = has2 ? LA.t[s2] : 0, i2 = has2 ? LA.idx[s2] : -2;
-                    auto count_le = [&](int x) {
-                        int lo = 0, hi = ccount;
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if (LC.t[mid] <= x) lo = mid + 1;
-                            else hi = mid;
-                        }
-                        return lo;
-                    };
-                    auto slot_of = [&](int j) {
-                        int lo = 0, hi = ccount;
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if (LC.idx[mid] < j) lo = mid + 1;
-                            else hi = mid;
-                        }
-                        return lo < ccount && LC.idx[lo] == j ? lo : -1;
-                    };
-                    const int pbs = slot_of(ib);
-                    const int nT = T > 0 ? count_le(tw - T) : 0;                  // c too far from the witness
-                    const int pw = slot_of(iw);                                   // c at the witness's point
-                    anybad = nT - (pbs >= 0 && pbs < nT ? 1 : 0) > 0 || pw >= 0;
-                    if (anybad) {
-                        if (!has2) {
-                            loose = true;
-                        } else {
-                            // a c that rules out both: too far from both, or at one's point and too far from
-                            // the other
-                            const int nT2 = T > 0 ? count_le(min(tw, t2) - T) : 0;
-                            const int p2 = slot_of(i2);
-                            loose = nT2 - (pbs >= 0 && pbs < nT2 ? 1 : 0) > 0 || (p2 >= 0 && p2 < nT) ||
-                                    (pw >= 0 && T > 0 && t2 - tw >= T);
-                        }
-                    }
+                    const int q = h & 1;
+                    const int32_t *arr = q == 0 ? LC.t : LC.idx;
+                    const int x = q == 0 ? (T > 0 ? min(tw, t2) - T + 1 : INT32_MIN) : i2;
+                    int f = lower_bound(arr, x);
+                    if (q == 1 && !(f < nc && arr[f] == x)) f = KM;
+                    const int nT2 = min(__shfl_sync(full, f, base_lane), ccount);
+                    const int p2 = __shfl_sync(full, f, base_lane + 1);
+                    // a c that rules out both: too far from both, or at one's point and too far from the other
+                    loose = !has2 || nT2 - (pbs < nT2 ? 1 : 0) > 0 || p2 < nT || (pw < ccount && T > 0 && t2 - tw >= T);
                 }
-                float thr = bv + gmax + 1e-6f * bv;
-                if (anybad) thr = !loose && m2 < kInf ? fmaxf(thr, m2 + gmax + 1e-6f * m2) : kInf;
-                // keep base <= thr, compacted in increasing a: positions from the pair's kept masks
-                unsigned long long mk = 0;
-                if (live) {
-#pragma unroll 8
-                    for (int k = k0; k < AH; ++k) {
-                        const float bs = arow[NP * k + h];   // +inf for a past the list
-                        if (bs < kInf && bs <= thr) mk |= 1ull << k;
-                    }
+                float thr = m1 + gmax + 1e-6f * m1;
+                if (anybad) thr = loose ? kInf : fmaxf(thr, m2 + gmax + 1e-6f * m2);
+                thr = live ? fminf(thr, 3.402823466e38f) : -kInf;   // no infeasible a, and none for a b without cells
+                // keep base <= thr, in increasing a: positions from the kept counts of the row's threads
+                unsigned mk = 0;
+#pragma unroll
+                for (int k = 0; k < AH; ++k)
+                    if (v[k] <= thr) mk |= 1u << k;
+                mk = ((mk << rot) | (mk >> (AH - rot))) & ((1u << AH) - 1);
+                int pos = 0, kept = __popc(mk);
+#pragma unroll
+                for (int off = 1; off < TPB; off <<= 1) {
+                    const int o = __shfl_xor_sync(full, kept, off);
+                    if (h & off) pos += o;
+                    kept += o;
                 }
-                unsigned long long pmk = 0;
-                if constexpr (NP == 2) pmk = __shfl_xor_sync(0xffffffffu, (unsigned)mk, 1);
-                const int kept = __popcll(mk) + __popcll(pmk);
-                float *fbf = reinterpret_cast<float *>(sm.fb);
-                for (unsigned long long m = mk; m; m &= m - 1) {
-                    const int k = __ffsll((long long)m) - 1;
-                    const int a = NP * k + h;
-                    int pos = __popcll(mk & ((1ull << k) - 1));
-                    if constexpr (NP == 2) pos += __popcll(pmk & ((h ? 2ull << k : 1ull << k) - 1));
-                    const int at = fb_at<KM>(b, pos);
+                for (unsigned m = mk; m; m &= m - 1, ++pos) {
+                    const int j = __ffs((int)m) - 1, a = AH * h + j;
                     const float2 pa = LA.xy[a];
-                    fbf[2 * at] = arow[a];
-                    sm.fs[fs_at<KM>(b, pos)] = (uint8_t)(a | (pa.x == pb.x && pa.y == pb.y ? 0x80 : 0));
-                    fbf[2 * at + 1] = wrap_pi(__fadd_rn(A1, direction(pb, pa)));   // p1 = A1 + theta(b->a)
+                    const bool same = pa.x == pb.x && pa.y == pb.y;
+                    if (same) sm.coin[i & 1] = 1;
+                    // p1 = A1 + theta(b->a)
+                    sm.fb[b * FS + pos] = make_float2(arow[j], wrap_pi(__fadd_rn(A1, direction(pb, pa))));
+                    sm.fs[b * SS + pos] = (uint8_t)(a | (same ? 0x80 : 0));
                 }
                 // tiles in decreasing kept count, then increasing b (the lanes of a warp then loop over
                 // similar numbers of a): b's first tile = sum of the tile counts of the b ranked before it
-                const int nt_b = inb ? (ccount + CT - 1) / CT : 0;
-                const int fnb = live ? kept : 0;
-                const int key = nt_b > 0 ? ((fnb + 1) << 8) | (255 - b) : 0;
                 if (h == 0) {
-                    sm.fn[b] = (uint8_t)fnb;
-                    sm.tcount[b] = (uint8_t)nt_b;
-                    sm.pw[b] = (key << 5) | nt_b;
+                    const int nt_b = (ccount + CT - 1) / CT;
+                    const int key = nt_b > 0 ? ((kept + 1) << 8) | (255 - b) : 0;
+                    sm.key(b) = (key << 5) | nt_b;
                 }
-            } else {
-                // ---- phase 2 (concurrent): theta(a->c) for every a and the c with t'(c) <= t'(a)
-                if (pf) {
-                    pf_n = ccnt[i - 3];
-                    pf_j = cidx[(int64_t)(i - 3) * K + pfi];
-                    pf_u = cu[(int64_t)(i - 3) * K + pfi];
+            }
+            if (pf && tid < pf_n) {
+                pf_xy = sc.xy[pf_j];
+                pf_t = sc.t[pf_j];
+            }
+            // ---- phase 2: theta(a->c) for every a and the c = row with t'(c) <= t'(a). A kept a of a cell (b, c) has
+            // t'(a) >= t'(b) >= t'(c), so only the rows from the first a with t'(a) >= t'(c) are read; entries of c
+            // past the list belong to cells whose theta(b->c) is +inf, so their value is never used either
+            if (row < nc) {
+                const int c = row;
+                const int tc = LC.t[c], ic = LC.idx[c];
+                const float2 pc = LC.xy[c];
+                int lo = 0;
+                for (int hi = na; lo < hi;) {
+                    const int mid = (lo + hi) >> 1;
+                    if (LA.t[mid] < tc) lo = mid + 1;
+                    else hi = mid;
                 }
-                if (tid == P1 && i >= 3) sm.geo[(i - 1) & 1] = md.geo[i - 1];
-                {
-                    // two threads per c, interleaved a. A kept a of a cell (b, c) has t'(a) >= t'(b) >= t'(c), so
-                    // only the rows from the first a with t'(a) >= t'(c) are read; entries of c past the list
-                    // belong to cells whose theta(b->c) is +inf, so their value is never used either
-                    const int q = tid - P1, c = q >> 1, h2 = q & 1;
-                    if (c < nc) {
-                        const int tc = LC.t[c], ic = LC.idx[c];
-                        const float2 pc = LC.xy[c];
-                        int lo = 0, hi = na;
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if (LA.t[mid] < tc) lo = mid + 1;
-                            else hi = mid;
-                        }
-                        for (int a = lo + h2; a < na; a += 2) {
-                            const int ta = LA.t[a];
-                            float r = kInf;
-                            if (!(T > 0 && ta - tc >= T) && LA.idx[a] != ic) r = direction(LA.xy[a], pc);   // theta(a->c)
-                            sm.r[a * RS + c] = r;
-                        }
-                    }
-                }
-                pf_ok = pf && pfi < pf_n;
-                if (pf_ok) {
-                    pf_xy = sc.xy[pf_j];
-                    pf_t = sc.t[pf_j];
+#pragma unroll 2
+                for (int a = lo + h; a < na; a += TPB) {
+                    const int ta = LA.t[a];
+                    float r = direction(LA.xy[a], pc);   // theta(a->c)
+                    if ((T > 0 && ta - tc >= T) || LA.idx[a] == ic) r = kInf;
+                    sm.r[a * RS + c] = r;
                 }
             }
             __syncthreads();
@@ -404,55 +381,53 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // tile layout, by every thread (NT / KM per b): b's first tile = the tile count of the b ranked
             // before it (decreasing kept count, then increasing b)
             {
-                constexpr int RP = NT / KM;
-                static_assert(RP >= 1 && RP <= 32 && (RP & (RP - 1)) == 0, "threads per b in the ranking");
-                const int b = tid / RP, part = tid % RP;
-                const int wb = sm.pw[b], key = wb >> 5, nt_b = wb & 31;
+                const int b = row, wb = sm.key(b), key = wb >> 5, nt_b = wb & 31;
                 int before = 0, total = 0;
-                for (int b2 = part; b2 < KM; b2 += RP) {
-                    const int w = sm.pw[b2];
+                for (int b2 = h; b2 < KM; b2 += TPB) {
+                    const int w = sm.key(b2);
                     total += w & 31;
                     if ((w >> 5) > key) before += w & 31;
                 }
 #pragma unroll
-                for (int off = 1; off < RP; off <<= 1) {
-                    before += __shfl_xor_sync(0xffffffffu, before, off);
-                    total += __shfl_xor_sync(0xffffffffu, total, off);
+                for (int off = 1; off < TPB; off <<= 1) {
+                    before += __shfl_xor_sync(full, before, off);
+                    total += __shfl_xor_sync(full, total, off);
                 }
-                if (part == 0) sm.tbase[b] = (uint16_t)before;
-                for (int t = part; t < nt_b; t += RP) sm.tile_b[before + t] = (uint8_t)b;
-                if (tid == 0) sm.ntile = total;
+                if (h == 0) sm.info(b) = before << 12 | max((key >> 8) - 1, 0) << 5 | nt_b;
+                for (int t = h; t < nt_b; t += TPB) sm.tile_b(before + t) = (uint8_t)b;
+                if (tid == 0) {
+                    sm.ntile = total;
+                    sm.coin[(i - 1) & 1] = 0;
+                }
             }
 
             // list A is not read from here on: its buffer receives list C of the next step
-            if (pf) {
-                LA.idx[pfi] = pf_ok ? pf_j : -1;
-                LA.xy[pfi] = pf_xy;
-                LA.t[pfi] = pf_t;
-                LA.u[pfi] = pf_ok ? pf_u : kInf;
-                if (pfi == 0) LA.n = pf_n;
-            }
-            if (i >= 3 && pfi >= K && pfi < KM) {
-                LA.idx[pfi] = -1;
-                LA.xy[pfi] = make_float2(0.f, 0.f);
-                LA.t[pfi] = 0x3fffffff;
-                LA.u[pfi] = kInf;
+            if (i >= 3 && tid < KM) {
+                const bool ok = tid < pf_n;
+                LA.idx[tid] = ok ? pf_j : -1;
+                LA.xy[tid] = pf_xy;
+                LA.t[tid] = pf_t;
+                LA.u[tid] = ok ? pf_u : kInf;
+                if (tid == 0) LA.n = pf_n;
             }
 
             __syncthreads();   // the tile layout is complete
 
             // ---- phase 3: tiles (b, CT consecutive c)
             const int ntile = sm.ntile;
+            const bool coin = sm.coin[i & 1] != 0;
             uint8_t *bstep = ubeta + (int64_t)(i - 2) * K * K;
             // tiles in decreasing kept count, dealt to the threads back and forth (round r: thread t takes
             // tile r NT + t for even r, r NT + NT - 1 - t for odd r) so that per-thread sums even out
             for (int r0 = 0; r0 < ntile; r0 += NT) {
                 const int tile = r0 + (((r0 / NT) & 1) ? NT - 1 - tid : tid);
                 if (tile >= ntile) continue;
-                const int b = sm.tile_b[tile];
-                const int c0 = (tile - sm.tbase[b]) * CT;
+                const int b = sm.tile_b(tile);
+                const int info = sm.info(b);
+                const int c0 = (tile - (info >> 12)) * CT;
                 const float2 pb = LB.xy[b];
                 const int tb = LB.t[b], ib = LB.idx[b];
+                const float ub = LB.u[b];
                 float q1[CT], best[CT];
                 int arg[CT], tcq[CT];
 #pragma unroll
@@ -468,30 +443,29 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     for (int k = 0; k < 4; ++k) {
                         const int c = c0 + q4 + k;
                         const bool ok = c < nc && tv[k] <= tb && iv[k] != ib;
-                        q1[q4 + k] = ok ? direction(pb, xv[k]) : kInf;   // theta(b->c)
+                        const float d = direction(pb, xv[k]);            // theta(b->c)
+                        q1[q4 + k] = ok ? d : kInf;
                         tcq[q4 + k] = tv[k];
                         best[q4 + k] = kInf;
                         arg[q4 + k] = kNoSlot;
                     }
                 }
-                const int nf = sm.fn[b];
+                const int nf = (info >> 5) & 127;
                 // cells in pairs: packed FP32x2 arithmetic, same roundings as triple_cost
                 static_assert(CT % 4 == 0, "tiles of a multiple of 4 cells");
                 unsigned long long q1p[CT / 2];
 #pragma unroll
                 for (int q = 0; q < CT / 2; ++q) q1p[q] = pk2(q1[2 * q], q1[2 * q + 1]);
                 const unsigned long long lamp = pk2(lam23, lam23);
-#pragma unroll UR
-                for (int k = 0; k < nf; ++k) {
-                    const float2 e = sm.fb[fb_at<KM>(b, k)];
-                    const int fa = sm.fs[fs_at<KM>(b, k)];
-                    const int a = fa & 0x7f;
-                    if constexpr (kCount) n_eval += CT;
-                    const float p2 = __fadd_rn(e.y, (fa & 0x80) ? k2c : k2);
+                const float2 *fb = sm.fb + b * FS;
+                const uint8_t *fs = sm.fs + b * SS;
+                const float *rc = sm.r + c0;
+                if constexpr (kCount) n_eval += CT * nf;
+                auto triples = [&](const float2 e, int a, float p2) {
                     const unsigned long long bp = pk2(e.x, e.x), p1p = pk2(e.y, e.y), p2p = pk2(p2, p2);
 #pragma unroll
                     for (int q4 = 0; q4 < CT; q4 += 4) {
-                        const float4 r4 = *reinterpret_cast<const float4 *>(&sm.r[a * RS + c0 + q4]);
+                        const float4 r4 = *reinterpret_cast<const float4 *>(rc + a * RS + q4);
                         float v[4];
                         triple_cost2(bp, p1p, p2p, q1p[q4 / 2], pk2(r4.x, r4.y), lamp, v[0], v[1]);
                         triple_cost2(bp, p1p, p2p, q1p[q4 / 2 + 1], pk2(r4.z, r4.w), lamp, v[2], v[3]);
@@ -499,24 +473,29 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                         for (int q = 0; q < 4; ++q)
                             if (v[q] < best[q4 + q]) { best[q4 + q] = v[q]; arg[q4 + q] = a; }
                     }
+                };
+                if (!coin) {
+#pragma unroll UR
+                    for (int k = 0; k < nf; ++k) triples(fb[k], fs[k], __fadd_rn(fb[k].y, k2));
+                } else {
+#pragma unroll 1
+                    for (int k = 0; k < nf; ++k)
+                        triples(fb[k], fs[k] & 0x7f, __fadd_rn(fb[k].y, (fs[k] & 0x80) ? k2c : k2));
                 }
                 // argmin bytes of the tile's cells, four at a time (c0 is a multiple of 4, and K, the row
                 // stride, is a multiple of 4 whenever a tile reaches past c0 + 3: the packed store is used
-                // only then)
+                // only then); a cell without a feasible a keeps best = +inf and arg = kNoSlot
                 uint32_t packed[CT / 4];
 #pragma unroll
                 for (int q4 = 0; q4 < CT / 4; ++q4) packed[q4] = 0;
 #pragma unroll
                 for (int q = 0; q < CT; ++q) {
                     const int c = c0 + q;
-                    float al = kInf;
-                    int bt = kNoSlot;
-                    if (best[q] < kInf) {
-                        al = cell_alpha(best[q], lam2, dt_bc, tb, tcq[q]);
-                        bt = arg[q];
-                    }
-                    if (c < nc) sm.alpha[c * AS + b] = al;
-                    packed[q / 4] |= (uint32_t)bt << (8 * (q % 4));
+                    // alpha_i(b,c), and before the last step the next step's base: U(b) and the same Delta with it
+                    const float al = cell_alpha(best[q], lam2, dt_bc, tb, tcq[q]);
+                    const float out = i > 2 ? base_cost(ub, lam2, dt_bc, tb, tcq[q], al) : al;
+                    if (c < nc) sm.alpha[c * AS + b] = out;
+                    packed[q / 4] |= (uint32_t)arg[q] << (8 * (q % 4));
                 }
                 const bool aligned = (K & 3) == 0;
 #pragma unroll
@@ -536,7 +515,7 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // infeasible there); only the initial pair search of Eq. 13 reads every cell of the last step
             if (i == 2) {
                 for (int b = warp; b < nb; b += NW) {
-                    const int covered = sm.tcount[b] * CT;
+                    const int covered = (sm.info(b) & 31) * CT;
                     for (int c = covered + lane; c < nc; c += 32) sm.alpha[c * AS + b] = kInf;
                 }
             }
@@ -589,17 +568,16 @@ struct FusedArgs {
     int32_t *assign = nullptr;
 };
 
-template <int KM, int NT, int CT, int NP, int UR, bool kCount, bool kFused>
+template <int KM, int NT, int MB, int CT, int UR, bool kCount, bool kFused>
 cudaError_t launch_recurse_t(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
                              Params p, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
                              uint8_t *beta, UnitResult *res, int *work_counter, unsigned long long *evaluated,
                              const FusedArgs &fa, cudaStream_t st)
 {
     // three CTAs of 256 threads per SM: 3 x (shared memory + 1 KB reserved) <= 228 KB
-    static_assert(KM != 64 || NT != 256 || 3 * (sizeof(Smem<KM, NT, NP>) + 1024) <= 228 * 1024,
-                  "recursion shared memory exceeds the three-CTA budget");
-    auto kern = recurse_kernel<KM, NT, CT, NP, UR, kCount, kFused>;
-    const size_t smem = sizeof(Smem<KM, NT, NP>);
+    static_assert(MB * (sizeof(Smem<KM, NT>) + 1024) <= 228 * 1024, "recursion shared memory exceeds the CTAs' budget");
+    auto kern = recurse_kernel<KM, NT, MB, CT, UR, kCount, kFused>;
+    const size_t smem = sizeof(Smem<KM, NT>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
@@ -626,18 +604,18 @@ cudaError_t dispatch(int variant, const Unit *units, int64_t n_units, const Mode
                      UnitResult *res, int *work_counter, unsigned long long *evaluated, const FusedArgs &fa,
                      cudaStream_t st)
 {
-#define HGM_RECURSE(KM_, NT_, CT_, NP_, UR_)                                                                      \
-    return launch_recurse_t<KM_, NT_, CT_, NP_, UR_, kCount, kFused>(units, n_units, models, scenes, p, cand_idx,  \
+#define HGM_RECURSE(KM_, NT_, MB_, CT_, UR_)                                                                      \
+    return launch_recurse_t<KM_, NT_, MB_, CT_, UR_, kCount, kFused>(units, n_units, models, scenes, p, cand_idx,  \
                                                                      cand_u, cand_cnt, beta, res, work_counter,   \
                                                                      evaluated, fa, st)
     if (p.K <= 32) {
-        if (variant == 1) HGM_RECURSE(32, 128, 8, 2, 2);
-        if (variant == 2) HGM_RECURSE(32, 128, 4, 2, 4);
-        HGM_RECURSE(32, 128, 4, 2, 2);
+        if (variant == 1) HGM_RECURSE(32, 128, 4, 8, 2);
+        if (variant == 2) HGM_RECURSE(32, 128, 4, 4, 4);
+        HGM_RECURSE(32, 128, 4, 4, 2);
     }
-    if (variant == 1) HGM_RECURSE(64, 256, 8, 2, 2);
-    if (variant == 2) HGM_RECURSE(64, 256, 4, 2, 4);
-    HGM_RECURSE(64, 256, 4, 2, 2);
+    if (variant == 1) HGM_RECURSE(64, 256, 3, 8, 2);
+    if (variant == 2) HGM_RECURSE(64, 256, 3, 4, 4);
+    HGM_RECURSE(64, 256, 3, 4, 2);
 #undef HGM_RECURSE
 }
 
@@ -673,12 +651,12 @@ cudaError_t launch_model_geo(const float2 *xy, const int32_t *t, int M, float4 *
 cudaError_t preload_recurse()
 {
     cudaFuncAttributes a;
-    const void *kerns[] = {(const void *)recurse_kernel<32, 128, 8, 2, 2, false, false>,
-                           (const void *)recurse_kernel<32, 128, 4, 2, 4, false, false>,
-                           (const void *)recurse_kernel<32, 128, 4, 2, 2, false, false>,
-                           (const void *)recurse_kernel<64, 256, 8, 2, 2, false, false>,
-                           (const void *)recurse_kernel<64, 256, 4, 2, 4, false, false>,
-                           (const void *)recurse_kernel<64, 256, 4, 2, 2, false, false>};
+    const void *kerns[] = {(const void *)recurse_kernel<32, 128, 4, 8, 2, false, false>,
+                           (const void *)recurse_kernel<32, 128, 4, 4, 4, false, false>,
+                           (const void *)recurse_kernel<32, 128, 4, 4, 2, false, false>,
+                           (const void *)recurse_kernel<64, 256, 3, 8, 2, false, false>,
+                           (const void *)recurse_kernel<64, 256, 3, 4, 4, false, false>,
+                           (const void *)recurse_kernel<64, 256, 3, 4, 2, false, false>};
     for (const void *k : kerns) {
         cudaError_t e = cudaFuncGetAttributes(&a, k);
         if (e != cudaSuccess) return e;

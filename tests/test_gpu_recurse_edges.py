@@ -1,0 +1,66 @@
+"""The recursion kernel at the edges of its lists: caps around the two table sizes and off the 4-cell tiles, lists
+shorter than the cap and of very different lengths, crowded frames (many points of equal time), every closeness
+limit, points shared between lists, small and large numbers of units. Against the FP64 oracle on every offset
+(tests/gpu_util.check_offset: energies 1e-5 relative, assignments equal or of the same FP64 energy)."""
+import numpy as np
+import pytest
+
+from gpu_util import check_offset
+from paper_1505_00581_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1505_00581_gb300 import build, hgm
+    build.build()
+    hgm.load()
+    import oracle
+    oracle.build()
+    return torch, hgm, oracle
+
+
+def _scene(rng, mod, n_frames, lam, crowd):
+    sc = synth.make_scene(rng, n_frames, (60.0, 40.0), ("poisson", lam), mod.centres, [mod], [(0, 2)])
+    t = sc.t.copy()
+    t[rng.random(len(t)) < crowd] = n_frames // 2
+    return synth.Scene(sc.xy, t, sc.f, None, n_frames, [])
+
+
+@pytest.mark.parametrize("K,lam,crowd,T,window,M", [
+    (17, 6.0, 0.0, 10, 2, 9), (31, 9.0, 0.2, 10, 3, 12), (32, 20.0, 0.0, 4, 2, 8), (33, 8.0, 0.1, 10, 2, 10),
+    (47, 20.0, 0.3, 10, 3, 7), (63, 30.0, 0.0, 0, 1, 6), (64, 4.0, 0.5, 10, 3, 11), (64, 30.0, 0.0, 2, 3, 9),
+    (64, 1.0, 0.0, 10, 3, 20), (61, 25.0, 0.1, 10, 2, 3)])
+def test_list_edges(env, K, lam, crowd, T, window, M):
+    torch, hgm, oracle = env
+    rng = np.random.default_rng(1000 * K + M)
+    mod = synth.make_model(rng, M, F=16, frame=(60.0, 40.0), t_span=10, T=max(T, 6))
+    sc = _scene(rng, mod, 26, lam, crowd)
+    m, s = hgm.Model(mod.xy, mod.t, mod.f), hgm.Scene(sc.xy, sc.t, sc.f, sc.n_frames)
+    p = hgm.default_params(K=K, window=window, T=T)
+    first, e, a = hgm.match(m, s, p)
+    orc = oracle.Oracle(mod.xy, mod.t, mod.f, sc.xy, sc.t, sc.f, sc.n_frames, K=K, window=window, T=T,
+                        lambda1=0.6, lambda2=0.2, lambda3=5.0)
+    for k in range(len(e)):
+        ok, _, why = check_offset(orc, first + k, e[k], a[k])
+        assert ok, (first + k, why)
+
+
+@pytest.mark.parametrize("K", [32, 64])
+def test_few_and_many_units_give_the_same_bits(env, K):
+    """One offset, some and thousands of units in a call (the launch shapes differ, results must not)."""
+    torch, hgm, oracle = env
+    rng = np.random.default_rng(K)
+    mod = synth.make_model(rng, 14, F=16, frame=(60.0, 40.0), t_span=10)
+    sc = _scene(rng, mod, 700, 12.0, 0.01)
+    m, s = hgm.Model(mod.xy, mod.t, mod.f), hgm.Scene(sc.xy, sc.t, sc.f, sc.n_frames)
+    first, e, a = hgm.match(m, s, hgm.default_params(K=K, window=3))
+    for lo, n in ((first, 1), (first + 100, 40), (first + 200, 160), (first + 5, 400)):
+        p = hgm.default_params(K=K, window=3, offset_lo=lo, offset_hi=lo + n - 1)
+        f1, e1, a1 = hgm.match(m, s, p)
+        assert f1 == lo and len(e1) == n
+        assert np.array_equal(e1, e[lo - first:lo - first + n]) and np.array_equal(a1, a[lo - first:lo - first + n])
