@@ -421,7 +421,9 @@ __global__ void __launch_bounds__(256) prop_rescore_kernel(const Unit *__restric
 }
 
 // Precision mode, fallback units: every candidate of their full lists gets its FP32 unary cost (the same
-// value as the FP32 table). Unit count read on the device; one CTA per unit at a time.
+// value as the FP32 table). Unit count read on the device; a unit's candidates are spread over the grid's y
+// dimension, so that a handful of units (the usual case) fills the chip: one CTA per unit took 700 us for one
+// unit of 256 lists.
 __global__ void __launch_bounds__(256) rescore_units_kernel(const Unit *__restrict__ units, int64_t n_max,
                                                             const int *__restrict__ n_dev,
                                                             const ModelRec *__restrict__ models,
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(256) rescore_units_kernel(const Unit *__restri
         const ModelRec md = models[un.model];
         const SceneRec sc = scenes[un.scene];
         const int64_t lbase = un.cand / K;
-        for (int e = threadIdx.x; e < md.M * K; e += blockDim.x) {
+        for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < md.M * K; e += gridDim.y * blockDim.x) {
             const int li = e / K, c = e - li * K;
             if (c >= cand_cnt[lbase + li]) continue;
             const int64_t o = un.cand + e;
@@ -560,8 +562,8 @@ cudaError_t launch_rescore_units(const Unit *units, int64_t n_max, const int *n_
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int64_t grid = std::min<int64_t>(n_max, (int64_t)sms * 8);
-    rescore_units_kernel<<<(unsigned)grid, 256, 0, st>>>(units, n_max, n_dev, models, scenes, p, cand_idx, cand_cnt,
+    const dim3 grid((unsigned)std::min<int64_t>(n_max, sms), 32);
+    rescore_units_kernel<<<grid, 256, 0, st>>>(units, n_max, n_dev, models, scenes, p, cand_idx, cand_cnt,
                                                          cand_u);
     return cudaGetLastError();
 }
