@@ -48,6 +48,9 @@
 // fetched from global memory during phase 1 and stored in the buffer of the list A, which phase 3 no longer reads,
 // so no step waits on a global load. Argmin bytes are written for the tiled cells only, a tile's four at once: the
 // cells past b's time prefix are never on a chain, so the backtrack never reads them.
+#include <algorithm>
+#include <climits>
+
 #include "backtrack.cuh"
 #include "recurse_common.cuh"
 
@@ -132,11 +135,12 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                const SceneRec *__restrict__ scenes, Params p, const int32_t *__restrict__ cand_idx,
                const float *__restrict__ cand_u, const int32_t *__restrict__ cand_cnt, uint8_t *__restrict__ beta,
                UnitResult *__restrict__ res, int *__restrict__ work_counter, unsigned long long *__restrict__ evaluated,
-               const int *__restrict__ n_dev, int64_t beta_cta, float *__restrict__ energy_out,
+               const int *__restrict__ n_dev, int n_from, int n_to, int64_t beta_cta, float *__restrict__ energy_out,
                int32_t *__restrict__ assign_out)
 {
     if constexpr (kFused) {
         const int64_t nd = *n_dev;
+        if (nd <= n_from || nd > n_to) return;   // the launch for the other range of counts takes it
         n_units = nd < n_units ? nd : n_units;
     }
     unsigned long long n_eval = 0;
@@ -563,6 +567,7 @@ constexpr int kFusedPerSm = 3;   // CTAs per SM of the fused variant (its argmin
 
 struct FusedArgs {
     const int *n_dev = nullptr;
+    int n_from = -1, n_to = INT32_MAX;   // counts this launch solves: n_from < n <= n_to
     int64_t beta_cta = 0;
     float *energy = nullptr;
     int32_t *assign = nullptr;
@@ -589,11 +594,11 @@ cudaError_t launch_recurse_t(const Unit *units, int64_t n_units, const ModelRec 
     if (grid > n_units) grid = n_units;
     if ((e = cudaMemsetAsync(work_counter, 0, sizeof(int), st)) != cudaSuccess) return e;
     prof_begin(kProfRecurse, st);
-    if (kFused) {   // the per-CTA scratch was sized for sms * kFusedPerSm CTAs
-        grid = std::min<int64_t>((int64_t)sms * kFusedPerSm, n_units);
-    }
+    if (kFused)   // the per-CTA scratch was sized for sms * kFusedPerSm CTAs
+        grid = std::min<int64_t>(std::min<int64_t>(grid, (int64_t)sms * kFusedPerSm), n_units);
     kern<<<(unsigned)grid, NT, smem, st>>>(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res,
-                                           work_counter, evaluated, fa.n_dev, fa.beta_cta, fa.energy, fa.assign);
+                                           work_counter, evaluated, fa.n_dev, fa.n_from, fa.n_to, fa.beta_cta, fa.energy,
+                                           fa.assign);
     prof_end(kProfRecurse, st);
     return cudaGetLastError();
 }
@@ -620,6 +625,31 @@ cudaError_t dispatch(int variant, const Unit *units, int64_t n_units, const Mode
 }
 
 int g_variant = 0;   // recursion variant: 0 = 4 c per tile, 1 = 8 c per tile, 2 = 4 c per tile, triple loop unrolled by 4
+
+// At most one unit per SM: twice the threads per unit. A step's phases are chains of dependent operations that
+// more threads per row and per tile round shorten (model of 30 points, 150 units against 153: K = 64 268 and 415 us,
+// K = 32 160 and 201 us); with two units on an SM the second one's warps already fill the gaps (271 units of K = 64:
+// 439 us with 512 threads each, 444 with 256).
+template <bool kFused>
+cudaError_t launch_wide(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes, Params p,
+                        const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt, uint8_t *beta,
+                        UnitResult *res, int *work_counter, const FusedArgs &fa, cudaStream_t st)
+{
+    if (p.K <= 32)
+        return launch_recurse_t<32, 256, 1, 4, 2, false, kFused>(units, n_units, models, scenes, p, cand_idx, cand_u,
+                                                                 cand_cnt, beta, res, work_counter, nullptr, fa, st);
+    return launch_recurse_t<64, 512, 1, 4, 2, false, kFused>(units, n_units, models, scenes, p, cand_idx, cand_u,
+                                                             cand_cnt, beta, res, work_counter, nullptr, fa, st);
+}
+
+int64_t wide_units()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return sms;
+}
 
 }  // namespace
 
@@ -656,7 +686,9 @@ cudaError_t preload_recurse()
                            (const void *)recurse_kernel<32, 128, 4, 4, 2, false, false>,
                            (const void *)recurse_kernel<64, 256, 3, 8, 2, false, false>,
                            (const void *)recurse_kernel<64, 256, 3, 4, 4, false, false>,
-                           (const void *)recurse_kernel<64, 256, 3, 4, 2, false, false>};
+                           (const void *)recurse_kernel<64, 256, 3, 4, 2, false, false>,
+                           (const void *)recurse_kernel<32, 256, 1, 4, 2, false, false>,
+                           (const void *)recurse_kernel<64, 512, 1, 4, 2, false, false>};
     for (const void *k : kerns) {
         cudaError_t e = cudaFuncGetAttributes(&a, k);
         if (e != cudaSuccess) return e;
@@ -675,6 +707,9 @@ cudaError_t launch_recurse(const Unit *units, int64_t n_units, const ModelRec *m
     if (n_units <= 0) return cudaSuccess;
     if (p.K <= 16)   // short lists (pruned form): one warp per unit
         return launch_recurse_small(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, st);
+    if (n_units <= wide_units())
+        return launch_wide<false>(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, work_counter,
+                                  FusedArgs{}, st);
     return dispatch<false, false>(g_variant, units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta,
                                   res, work_counter, nullptr, FusedArgs{}, st);
 }
@@ -700,6 +735,14 @@ cudaError_t launch_recurse_fused(const Unit *units, int64_t n_max, const int *n_
     fa.beta_cta = ((int64_t)std::max(max_M - 2, 1) * p.K * p.K + 255) / 256 * 256;
     fa.energy = energy;
     fa.assign = assign;
+    // the count is known on the device only: one launch for few units, one for more (an idle one costs 2-3 us)
+    const int few = (int)std::min<int64_t>(wide_units(), INT32_MAX);
+    fa.n_to = few;
+    cudaError_t e = launch_wide<true>(units, std::min<int64_t>(n_max, few), models, scenes, p, cand_idx, cand_u, cand_cnt,
+                                      scratch, nullptr, work_counter, fa, st);
+    if (e != cudaSuccess || n_max <= few) return e;
+    fa.n_from = few;
+    fa.n_to = INT32_MAX;
     return dispatch<false, true>(0, units, n_max, models, scenes, p, cand_idx, cand_u, cand_cnt, scratch, nullptr,
                                  work_counter, nullptr, fa, st);
 }
