@@ -542,21 +542,16 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                 argmin_merge(bv, bk, __shfl_xor_sync(0xffffffffu, bv, off), __shfl_xor_sync(0xffffffffu, bk, off));
             if (lane == 0) { sm.red_v[warp] = bv; sm.red_k[warp] = bk; }
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0) {
+                // every lane merges the warps' results: the same values
+                bv = sm.red_v[0];
+                bk = sm.red_k[0];
                 for (int w = 1; w < NW; ++w) argmin_merge(bv, bk, sm.red_v[w], sm.red_k[w]);
-                UnitResult r;
-                r.pad = 0;
-                if (bv < kInf) {
-                    r.energy = bv;
-                    r.z1 = bk / KM;
-                    r.z2 = bk % KM;
-                } else {
-                    r.energy = kInf;
-                    r.z1 = -1;
-                    r.z2 = -1;
-                }
-                if constexpr (kFused) backtrack_unit(un, md, sc, K, cidx, ubeta, r, energy_out, assign_out);
-                else res[u] = r;
+                const bool ok = bv < kInf;
+                const int z1 = ok ? bk / KM : -1, z2 = ok ? bk % KM : -1;
+                if constexpr (kFused)
+                    backtrack_unit(un, md, sc, K, cidx, ubeta, ok ? bv : kInf, z1, z2, energy_out, assign_out, lane);
+                else if (lane == 0) res[u] = UnitResult{ok ? bv : kInf, z1, z2, 0};
             }
             __syncthreads();
         }
