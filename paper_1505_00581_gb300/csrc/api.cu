@@ -287,6 +287,31 @@ __global__ void gather_rows_kernel(const float *__restrict__ src, int F, const i
     if (nonfinite) atomicOr(bad, 1);
 }
 
+// The models' sorted rows one after another (model m's at row urow): descriptors of F floats (a multiple of 4) and,
+// if oxy is given, positions. One launch for all models: a copy per model cost 2-3 us of launch each.
+__global__ void gather_models_kernel(const ModelRec *__restrict__ models, int n, int F, float4 *__restrict__ of,
+                                     float2 *__restrict__ oxy)
+{
+    for (int m = blockIdx.y; m < n; m += gridDim.y) {
+        const ModelRec md = models[m];
+        const int per = F / 4;
+        const float4 *src = reinterpret_cast<const float4 *>(md.f);
+        float4 *dst = of + (int64_t)md.urow * per;
+        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < md.M * per; e += gridDim.x * blockDim.x) dst[e] = src[e];
+        if (oxy)
+            for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < md.M; e += gridDim.x * blockDim.x)
+                oxy[md.urow + e] = md.xy[e];
+    }
+}
+
+cudaError_t launch_gather_models(const ModelRec *models, int n, int F, float *of, float2 *oxy, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    gather_models_kernel<<<dim3(8, (unsigned)std::min(n, 65535)), 256, 0, st>>>(models, n, F, reinterpret_cast<float4 *>(of),
+                                                                             oxy);
+    return cudaGetLastError();
+}
+
 // Sorted, padded device copy of a descriptor array (host or device, n x F row-major): the raw rows go to the
 // device in one copy (none for device input), then a gather kernel applies the permutation. Returns
 // HGM_EINVAL on a non-finite component. Synchronous on st.
@@ -651,17 +676,26 @@ hgm_status run_batch(Exec &ex, const hgm_model *const *models, int nm, const hgm
         tmin_all = std::min(tmin_all, models[m]->t_sorted.front());
         tmax_all = std::max(tmax_all, models[m]->t_sorted.back());
     }
-    CK(ws.modelcat.ensure((size_t)R * F * sizeof(float)), "workspace (models)");
-    for (int m = 0; m < nm; ++m)
-        CK(cudaMemcpyAsync(ws.modelcat.as<float>() + (size_t)urow[m] * F, models[m]->d.f,
-                           (size_t)models[m]->d.M * F * sizeof(float), cudaMemcpyDeviceToDevice, st),
-           "gather model descriptors");
     std::vector<ModelRec> mrec(nm);
     for (int m = 0; m < nm; ++m)
         mrec[m] = ModelRec{models[m]->d.xy, models[m]->d.t, models[m]->d.perm, models[m]->d.M, urow[m],
                            models[m]->d.f, models[m]->d.geo};
     CK(ws.mrec.ensure(nm * sizeof(ModelRec)), "workspace");
     if ((rc = h2d(ex, ws.mrec.p, mrec.data(), nm * sizeof(ModelRec), st))) return rc;
+    // the models' rows: a single model's as they are, several gathered into one block
+    const float *model_f = models[0]->d.f;
+    const float2 *model_xy = models[0]->d.xy;
+    if (nm > 1) {
+        CK(ws.modelcat.ensure((size_t)R * F * sizeof(float)), "workspace (models)");
+        float2 *oxy = nullptr;
+        if (hp->prune) {
+            CK(ws.modelxy.ensure((size_t)R * 2 * sizeof(float)), "workspace (models)");
+            oxy = ws.modelxy.as<float2>();
+        }
+        CK(launch_gather_models(ws.mrec.as<ModelRec>(), nm, F, ws.modelcat.as<float>(), oxy, st), "gather models");
+        model_f = ws.modelcat.as<float>();
+        model_xy = oxy;
+    }
     CK(ws.status.ensure(sizeof(int)), "workspace");
     CK(cudaMemsetAsync(ws.status.p, 0, sizeof(int), st), "memset");
 
@@ -676,17 +710,12 @@ hgm_status run_batch(Exec &ex, const hgm_model *const *models, int nm, const hgm
                                          prop->L.F, Fu);
         const float *th = prop->theta;
         CK(ws.P.ensure((size_t)R * kPropHidden * sizeof(float)), "workspace (projections)");
-        CK(launch_rowdot_plain(ws.modelcat.as<float>(), R, F, th + prop->L.o_W1, kPropHidden, prop->L.dp, Fu,
+        CK(launch_rowdot_plain(model_f, R, F, th + prop->L.o_W1, kPropHidden, prop->L.dp, Fu,
                                th + prop->L.o_b1, ws.P.as<float>(), kPropHidden, ws.status.as<int>(), st),
            "projection kernel");
         // position terms of the model points folded into P (the scene points' into Q)
-        CK(ws.modelxy.ensure((size_t)R * 2 * sizeof(float)), "workspace (models)");
-        for (int m = 0; m < nm; ++m)
-            CK(cudaMemcpyAsync(ws.modelxy.as<float>() + (size_t)urow[m] * 2, models[m]->d.xy,
-                               (size_t)models[m]->d.M * 2 * sizeof(float), cudaMemcpyDeviceToDevice, st),
-               "gather model positions");
         CK(ws.Pb.ensure((size_t)R * kPropHidden * sizeof(__nv_bfloat16)), "workspace (projections)");
-        CK(launch_prop_fold_xy(ws.P.as<float>(), R, ws.modelxy.as<float>(), th + prop->L.o_W1 + 2 * Fu,
+        CK(launch_prop_fold_xy(ws.P.as<float>(), R, reinterpret_cast<const float *>(model_xy), th + prop->L.o_W1 + 2 * Fu,
                                prop->L.dp, -1.0f, ws.Pb.as<__nv_bfloat16>(), st),
            "projection kernel");
         pi.Pb = ws.Pb.as<__nv_bfloat16>();
@@ -709,7 +738,7 @@ hgm_status run_batch(Exec &ex, const hgm_model *const *models, int nm, const hgm
     ex.tensor = pruning || hp->precision == 1;
     if (hp->precision == 1) {
         CK(ws.mnorm.ensure((size_t)R * sizeof(float)), "workspace (norms)");
-        CK(launch_sqnorm_bf16(ws.modelcat.as<float>(), R, F, F, ws.mnorm.as<float>(), st), "norm kernel");
+        CK(launch_sqnorm_bf16(model_f, R, F, F, ws.mnorm.as<float>(), st), "norm kernel");
     }
 
     // outputs: device pointers are written in place, host ones through staging
@@ -821,12 +850,12 @@ hgm_status run_batch(Exec &ex, const hgm_model *const *models, int nm, const hgm
             float *U = const_cast<float *>(srec[(size_t)g].U);
             if (hp->precision == 1) {
                 CK(launch_sqnorm_bf16(segf, pts, F, F, ws.snorm.as<float>(), st), "norm kernel");
-                CK(launch_unary_bf16(ws.modelcat.as<float>(), R, segf, pts, F, F, ws.mnorm.as<float>(),
+                CK(launch_unary_bf16(model_f, R, segf, pts, F, F, ws.mnorm.as<float>(),
                                      ws.snorm.as<float>(), p.lambda1, U, srec[(size_t)g].upitch,
                                      ws.status.as<int>(), ws.ubf.p, ws.ubf.bytes, st),
                    "BF16 unary kernel");
             } else {
-                CK(launch_unary(ws.modelcat.as<float>(), R, segf, pts, F, p.lambda1, U, (int)srec[(size_t)g].upitch,
+                CK(launch_unary(model_f, R, segf, pts, F, p.lambda1, U, (int)srec[(size_t)g].upitch,
                                 st),
                    "unary kernel");
             }
@@ -1631,13 +1660,13 @@ hgm_status prep_block_models(BlockBufs &bb, const hgm_model *const *models, int 
     std::vector<ModelRec> mrec((size_t)nm);
     for (int m = 0; m < nm; ++m) {
         const hgm_model *md = models[m];
-        CK(cudaMemcpyAsync(bb.model.as<float>() + (size_t)bb.urow[(size_t)m] * Fp, md->d.f,
-                           (size_t)md->d.M * Fp * sizeof(float), cudaMemcpyDeviceToDevice, st),
-           "gather model descriptors");
         mrec[(size_t)m] = ModelRec{md->d.xy, md->d.t, md->d.perm, md->d.M, bb.urow[(size_t)m], md->d.f, md->d.geo};
     }
     Exec ex;
-    return h2d(ex, bb.mrec.p, mrec.data(), mrec.size() * sizeof(ModelRec), st);
+    hgm_status rc = h2d(ex, bb.mrec.p, mrec.data(), mrec.size() * sizeof(ModelRec), st);
+    if (rc) return rc;
+    CK(launch_gather_models(bb.mrec.as<ModelRec>(), nm, Fp, bb.model.as<float>(), nullptr, st), "gather models");
+    return HGM_OK;
 }
 
 // The whole-block problem for every (model, scene) pair; the models were prepared by prep_block_models.
