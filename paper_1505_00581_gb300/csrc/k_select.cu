@@ -7,16 +7,16 @@
 // the smallest unary cost are kept (ties to the lower scene index), and the
 // kept points are listed in ascending scene index (hence ascending frame).
 //
-// One warp per (unit, i). The K-th smallest key is found exactly by a radix
-// select on the IEEE bit patterns (unary costs are >= 0, so the bit pattern
-// orders like the value), one 8-bit digit per pass from the top; a final
-// ballot pass keeps every key below the threshold plus the first equal ones in
-// index order. Integer decisions therefore depend only on the FP32 keys of
-// kernel (a), bit for bit. The costs of one window share their top bits (same
-// exponent range), so the digits on which all keys agree are read off an AND
-// and an OR of the keys instead of being histogrammed: the first pass that
-// would otherwise put every key into one shared-memory bin -- 32 lanes adding
-// to the same counter, serialised -- is skipped.
+// One warp per (unit, i). The K-th smallest key is found exactly on the IEEE bit patterns (unary costs are >= 0, so
+// the bit pattern orders like the value): 256 equal bins between the window's smallest and largest key, the bin that
+// holds rank K, and so on inside it, until the bin is kept whole, holds one value, or the rank is one of its first
+// few values, which a warp-wide minimum finds. Costs of a window fill such bins evenly, so one or two rounds decide
+// (digits of the bit pattern took three or four, their first one with most keys in a few bins). A final ballot
+// pass keeps every key up to that value; only where some of its equals must go does it rank them in index order.
+// Integer decisions therefore depend only on the FP32 keys of kernel (a), bit for bit.
+// Measured with the digit passes and with this: windows of 210 keys (204,000 lists) 386 -> 202 us, of 560 keys
+// (522,000 lists) 1,602 -> 868 us, of 420 with the re-score (237,000 lists) 1,139 -> 651 us, of which the re-score,
+// four lists of eight at a time instead of eight lanes of a warp, about a third.
 #include "hgm_internal.cuh"
 #include "unary_common.cuh"
 
@@ -32,6 +32,10 @@ __device__ __forceinline__ uint32_t lanemask_lt()
     return m;
 }
 
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kRescoreMax = kRescore;   // candidates of a list re-scored in the precision mode
+static_assert(32 % kRescoreMax == 0, "whole lists fill a warp");
+
 // kKeyRegs keys per lane are held in registers: windows of up to 32 kKeyRegs keys are selected from them,
 // longer ones from memory in every pass. The launch picks 8 (three CTAs per SM) when the call's typical
 // window (the scenes' mean density over 2w+1 frames) fits 256 keys, else 20 (two CTAs per SM, the registers
@@ -44,14 +48,25 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) select_kernel(const U
                                                              float *__restrict__ cand_u,
                                                              int32_t *__restrict__ cand_cnt)
 {
-    __shared__ uint32_t hist[kWarps][256];
+    __shared__ __align__(16) uint32_t hist[kWarps][256];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int K = p.K;
+    const uint32_t lt_mask = lanemask_lt();
     for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
         const Unit un = units[u];
         const ModelRec md = models[un.model];
         const SceneRec sc = scenes[un.scene];
+        // precision mode: the re-scores of up to four lists wait until they fill the warp
+        int pend = 0, pend_i = 0, pend_slot = -1;
+        auto rescore = [&] {
+            if (pend_slot >= 0) {
+                const int64_t o = un.cand + (int64_t)pend_i * K + pend_slot;
+                cand_u[o] = unary_fp32(md.f + (int64_t)pend_i * p.F, sc.f + (int64_t)cand_idx[o] * p.F, p.F, p.lambda1);
+            }
+            pend = 0;
+            pend_slot = -1;
+        };
         for (int i = warp; i < md.M; i += kWarps) {
             int32_t *oidx = cand_idx + un.cand + (int64_t)i * K;
             float *ou = cand_u + un.cand + (int64_t)i * K;
@@ -72,8 +87,9 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) select_kernel(const U
                     ou[e] = e < n ? key[e] : __int_as_float(0x7f800000);
                 }
             } else {
-                // radix select of the K-th smallest key (1-based rank kk); windows of up to 32 kKeyRegs keys are
-                // read once into registers (lane + 32 q), longer ones from memory in every pass
+                // windows of up to 32 kKeyRegs keys are read once into registers (lane + 32 q), longer ones from
+                // memory in every pass; slots past the window hold 0xffffffff, above every key (costs are >= 0, so
+                // bit 31 of a key is clear)
                 const bool inreg = n <= 32 * kKeyRegs;
                 uint32_t kb[kKeyRegs];
 #pragma unroll
@@ -81,106 +97,115 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) select_kernel(const U
                     const int e = lane + 32 * q;
                     kb[q] = inreg && e < n ? __float_as_uint(key[e]) : 0xffffffffu;
                 }
-                // bits on which every key of the window agrees
-                uint32_t kand = 0xffffffffu, kor = 0u;
-                if (inreg) {
-#pragma unroll
-                    for (int q = 0; q < kKeyRegs; ++q)
-                        if (lane + 32 * q < n) { kand &= kb[q]; kor |= kb[q]; }
-                } else {
-                    for (int e = lane; e < n; e += 32) {
-                        const uint32_t b = __float_as_uint(key[e]);
-                        kand &= b;
-                        kor |= b;
-                    }
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    kand &= __shfl_xor_sync(0xffffffffu, kand, off);
-                    kor |= __shfl_xor_sync(0xffffffffu, kor, off);
-                }
-                const uint32_t differ = kand ^ kor;
-                uint32_t prefix = 0, mask = 0;
-                int kk = K;
-                for (int shift = 24; shift >= 0; shift -= 8) {
-                    if (((differ >> shift) & 255u) == 0) {   // one digit value for every key: no histogram
-                        prefix |= kand & (255u << shift);
-                        mask |= 255u << shift;
-                        continue;
-                    }
-                    for (int d = lane; d < 256; d += 32) hist[warp][d] = 0;
-                    __syncwarp();
+                auto each = [&](auto f) {
                     if (inreg) {
-                        // slots past the window hold 0xffffffff: costs are >= 0 (bit 31 clear), so such a slot
-                        // either fails the prefix test or lands in bin 255, above every real key's bin
 #pragma unroll
                         for (int q = 0; q < kKeyRegs; ++q) {
-                            const uint32_t b = kb[q];
-                            if ((b & mask) == prefix) atomicAdd(&hist[warp][(b >> shift) & 255u], 1u);
+                            if (q % 4 == 0 && 32 * q >= n) break;   // slots past the window are harmless
+                            f(kb[q], lane + 32 * q);
                         }
                     } else {
-                        for (int e = lane; e < n; e += 32) {
-                            uint32_t b = __float_as_uint(key[e]);
-                            if ((b & mask) == prefix) atomicAdd(&hist[warp][(b >> shift) & 255u], 1u);
-                        }
+                        for (int c0 = 0; c0 < n; c0 += 32)
+                            f(c0 + lane < n ? __float_as_uint(key[c0 + lane]) : 0xffffffffu, c0 + lane);
                     }
+                };
+                uint32_t lo = 0xffffffffu, hi = 0;
+                each([&](uint32_t b, int e) {
+                    lo = min(lo, b);
+                    hi = max(hi, e < n ? b : 0u);
+                });
+                lo = __reduce_min_sync(kFull, lo);
+                hi = __reduce_max_sync(kFull, hi);
+                // the kk-th smallest of the c keys in [lo, hi]; every key below lo is kept. Ends with tau: keys < tau
+                // are kept, and the first kk of the neq keys == tau
+                int kk = K, c = n, neq = 0;
+                uint32_t tau = 0;
+                for (;;) {
+                    if (kk == c || lo == hi) {   // the whole range, or a range of equals
+                        tau = hi;
+                        neq = c;
+                        break;
+                    }
+                    if (kk <= 2) {               // one of the range's two smallest values
+                        bool done = false;
+                        for (uint32_t from = lo; !done;) {
+                            uint32_t t = 0xffffffffu;
+                            each([&](uint32_t b, int) { t = min(t, b >= from ? b : 0xffffffffu); });
+                            t = __reduce_min_sync(kFull, t);
+                            int cnt = 0;
+                            each([&](uint32_t b, int) { cnt += b == t; });
+                            cnt = (int)__reduce_add_sync(kFull, (unsigned)cnt);
+                            if (cnt >= kk) {
+                                tau = t;
+                                neq = cnt;
+                                done = true;
+                            } else {
+                                kk -= cnt;
+                                from = t + 1;
+                            }
+                        }
+                        break;
+                    }
+                    const int shift = max(0, 24 - __clz((int)(hi - lo)));   // (hi - lo) >> shift < 256
+                    uint4 *h4 = reinterpret_cast<uint4 *>(hist[warp]) + 2 * lane;
+                    h4[0] = h4[1] = make_uint4(0, 0, 0, 0);
                     __syncwarp();
-                    uint32_t c[8];
+                    each([&](uint32_t b, int) {
+                        if (b >= lo && b <= hi) atomicAdd(&hist[warp][(b - lo) >> shift], 1u);
+                    });
+                    __syncwarp();
+                    const uint4 x = h4[0], y = h4[1];
+                    const uint32_t cn[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
                     uint32_t sum = 0;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) { c[q] = hist[warp][lane * 8 + q]; sum += c[q]; }
+                    for (int q = 0; q < 8; ++q) sum += cn[q];
                     uint32_t incl = sum;
 #pragma unroll
                     for (int off = 1; off < 32; off <<= 1) {
-                        uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+                        const uint32_t v = __shfl_up_sync(kFull, incl, off);
                         if (lane >= off) incl += v;
                     }
-                    uint32_t excl = incl - sum;
-                    bool mine = excl < (uint32_t)kk && (uint32_t)kk <= incl;
-                    int digit = 0;
-                    uint32_t below = excl;
-                    if (mine) {
+                    const bool mine = incl - sum < (uint32_t)kk && (uint32_t)kk <= incl;
+                    uint32_t below = incl - sum, in_bin = 0;
+                    int bin = 0;
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            if (below + c[q] >= (uint32_t)kk) { digit = lane * 8 + q; break; }
-                            below += c[q];
+                    for (int q = 0; q < 8; ++q) {
+                        const bool here = in_bin == 0 && below + cn[q] >= (uint32_t)kk;
+                        if (here) {
+                            bin = lane * 8 + q;
+                            in_bin = cn[q];
+                        } else if (in_bin == 0) {
+                            below += cn[q];
                         }
                     }
-                    uint32_t ball = __ballot_sync(0xffffffffu, mine);
-                    int src = __ffs(ball) - 1;
-                    digit = __shfl_sync(0xffffffffu, digit, src);
-                    below = __shfl_sync(0xffffffffu, below, src);
-                    prefix |= (uint32_t)digit << shift;
-                    mask |= 255u << shift;
-                    kk -= (int)below;
+                    const int src = __ffs((int)__ballot_sync(kFull, mine)) - 1;
+                    bin = __shfl_sync(kFull, bin, src);
+                    kk -= (int)__shfl_sync(kFull, below, src);
+                    c = (int)__shfl_sync(kFull, in_bin, src);
+                    lo += (uint32_t)bin << shift;
+                    hi = min(hi, lo + ((1u << shift) - 1));
                     __syncwarp();
                 }
-                // keep keys < tau, plus the first kk keys == tau in index order (tau is a real key's bits, so
-                // the 0xffffffff of slots past the window is never kept)
-                const uint32_t tau = prefix;
-                const uint32_t lt_mask = lanemask_lt();
-                int base = 0, eqseen = 0;
-                auto keep_step = [&](uint32_t b, int e) {
-                    const bool lt = b < tau;
-                    const bool eq = b == tau;
-                    const uint32_t eqm = __ballot_sync(0xffffffffu, eq);
-                    const int eqrank = eqseen + __popc(eqm & lt_mask);
-                    const bool keep = lt || (eq && eqrank < kk);
-                    const uint32_t km = __ballot_sync(0xffffffffu, keep);
-                    const int pos = base + __popc(km & lt_mask);
-                    if (keep && pos < K) { oidx[pos] = j0 + e; ou[pos] = __uint_as_float(b); }
-                    base += __popc(km);
-                    eqseen += __popc(eqm);
-                };
-                if (inreg) {
-#pragma unroll
-                    for (int q = 0; q < kKeyRegs; ++q)
-                        if (32 * q < n) keep_step(kb[q], lane + 32 * q);
-                } else {
-                    for (int c0 = 0; c0 < n; c0 += 32) {
-                        const int e = c0 + lane;
-                        keep_step(e < n ? __float_as_uint(key[e]) : 0xffffffffu, e);
+                // keep keys < tau, plus the first kk keys == tau in index order
+                int base = 0;
+                auto put = [&](bool keep, uint32_t b, int e) {
+                    const uint32_t km = __ballot_sync(kFull, keep);
+                    if (keep) {
+                        const int pos = base + __popc(km & lt_mask);
+                        oidx[pos] = j0 + e;
+                        ou[pos] = __uint_as_float(b);
                     }
+                    base += __popc(km);
+                };
+                if (kk == neq) {
+                    each([&](uint32_t b, int e) { put(b <= tau, b, e); });
+                } else {
+                    int eqseen = 0;
+                    each([&](uint32_t b, int e) {
+                        const uint32_t eqm = __ballot_sync(kFull, b == tau);
+                        put(b < tau || (b == tau && eqseen + __popc(eqm & lt_mask) < kk), b, e);
+                        eqseen += __popc(eqm);
+                    });
                 }
             }
             if (lane == 0) cand_cnt[un.cand / K + i] = kept;
@@ -188,29 +213,24 @@ __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) select_kernel(const U
                 // precision mode: the p.rescore smallest approximate costs (ties: lower slot) are
                 // recomputed from the FP32 descriptors in the exact kernel's fixed FMA order
                 __syncwarp();
-                float kv[2];
-                kv[0] = lane < kept ? ou[lane] : __int_as_float(0x7f800000);
-                kv[1] = lane + 32 < kept ? ou[lane + 32] : __int_as_float(0x7f800000);
-                int mine = -1;
-                const int rounds = p.rescore < kept ? p.rescore : kept;
+                uint32_t k0 = lane < kept ? __float_as_uint(ou[lane]) : 0xffffffffu;
+                uint32_t k1 = lane + 32 < kept ? __float_as_uint(ou[lane + 32]) : 0xffffffffu;
+                const int rounds = min(min(p.rescore, kRescoreMax), kept);
                 for (int q = 0; q < rounds; ++q) {
-                    float bv = kv[0] <= kv[1] ? kv[0] : kv[1];
-                    int bs = kv[0] <= kv[1] ? lane : lane + 32;
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-                        const int os = __shfl_xor_sync(0xffffffffu, bs, off);
-                        if (ov < bv || (ov == bv && os < bs)) { bv = ov; bs = os; }
+                    const uint32_t m = __reduce_min_sync(kFull, min(k0, k1));
+                    const uint32_t e0 = __ballot_sync(kFull, k0 == m), e1 = __ballot_sync(kFull, k1 == m);
+                    const int slot = e0 ? __ffs((int)e0) - 1 : 31 + __ffs((int)e1);
+                    if (lane == kRescoreMax * pend + q) {
+                        pend_slot = slot;
+                        pend_i = i;
                     }
-                    if (lane == q) mine = bs;
-                    if (bs == lane) kv[0] = __int_as_float(0x7f800000);
-                    if (bs == lane + 32) kv[1] = __int_as_float(0x7f800000);
+                    if (slot == lane) k0 = 0xffffffffu;
+                    if (slot == lane + 32) k1 = 0xffffffffu;
                 }
-                if (mine >= 0 && mine < kept) {
-                    ou[mine] = unary_fp32(md.f + (int64_t)i * p.F, sc.f + (int64_t)oidx[mine] * p.F, p.F, p.lambda1);
-                }
+                if (++pend == 32 / kRescoreMax) rescore();
             }
         }
+        if (pend) rescore();
     }
 }
 
