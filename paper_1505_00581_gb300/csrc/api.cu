@@ -604,7 +604,7 @@ hgm_status run_units(Exec &ex, const hgm_model *const *models, std::vector<Unit>
         }
         if (p.dummy >= 0) {
             // the dummy assignment: its own recursion kernel, which also backtracks
-            const int grid = dummy_grid();
+            const int grid = dummy_grid(K);
             if (grid <= 0) return fail(HGM_ECUDA, "device query failed");
             CK(ws.beta_dummy.ensure((size_t)dummy_scratch_bytes(K, max_M, grid)), "workspace (argmin tables)");
             unsigned long long *ev = nullptr;
@@ -613,8 +613,8 @@ hgm_status run_units(Exec &ex, const hgm_model *const *models, std::vector<Unit>
                 ev = ws.evaluated.as<unsigned long long>();
             }
             CK(launch_recurse_dummy(du, n, dm, ds, p, p.dummy, ws.cand_idx.as<int32_t>(), ws.cand_u.as<float>(),
-                                    ws.cand_cnt.as<int32_t>(), ws.beta_dummy.as<uint8_t>(), max_M, grid, d_energy,
-                                    d_assign, ev, st),
+                                    ws.cand_cnt.as<int32_t>(), ws.beta_dummy.as<uint8_t>(), max_M, grid,
+                                    ws.counter.as<int>(), d_energy, d_assign, ev, st),
                "recursion kernel (dummy)");
             begin = end;
             continue;

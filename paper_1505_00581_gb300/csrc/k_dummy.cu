@@ -1,92 +1,92 @@
 // k_dummy.cu -- the recursion with the dummy assignment of Eq. 2 (reading R5).
 //
-// Every candidate list C_i(o) gets one more slot, eps, after its real candidates (slot K of a table of
-// L = K + 1 slots), with U(eps) = lambda1 W^d. A term that involves eps vanishes (Delta(i,j) if z_i or
-// z_j is eps; D^g if any point of the triangle is), and a triple holding eps is feasible iff its real
-// points, in chain order, are distinct, time-ordered and less than T frames apart. So the all-eps chain
-// is always feasible and every offset has a finite optimum.
+// Every candidate list C_i(o) gets one more slot, eps, after its real candidates, with U(eps) = lambda1 W^d. A term
+// that involves eps vanishes (Delta(i,j) if z_i or z_j is eps; D^g if any point of the triangle is), and a triple
+// holding eps is feasible iff its real points, in chain order, are distinct, time-ordered and less than T frames
+// apart. So the all-eps chain is always feasible and every offset has a finite optimum.
 //
-// One persistent CTA per unit, all tables in shared memory (L x L floats each): alpha_{i+1} and alpha_i
-// (ping-pong), base(b, a) = U(a) + lambda2 Delta(a, b) + alpha_{i+1}(a, b) (eps rules applied), and the
-// per-step directions P1(b, a) = A1 + theta(b->a), P2(b, a) = A2 + theta(a->b) (kept pairs only),
-// R(a, c) = theta(a->c) (only for the a some row keeps, once the kept lists are built).
-// Every open cell (b, c) has a best of at most thr(b): base(b, eps), since the triple (eps, b, c) is
-// feasible and costs that alone, and base(b, a1) + max D^g when the row's smallest base a1 is feasible with
-// every open c. A warp per row keeps the a with base <= thr(b) that may follow b and ranks them by
-// (base, slot). Threads take groups of four consecutive c of one b (c fastest, so a warp shares b:
-// broadcast reads of base, P1, P2) and walk b's kept a in that order until no open cell of the group can
-// improve. The argmin slots go to a per-CTA global scratch, (M-2) x L x L bytes, and the CTA backtracks
-// its own unit (Eq. 12); eps is reported as -2 in the assignment.
+// The real cells (b, c) run as in k_recurse.cu (its comments hold here: row lists from registers, tiles of four c of
+// one b in decreasing kept count, the next step's base written with alpha), with three differences:
+//  * a cell starts from the triple (eps, b, c), which is feasible and costs base(eps, b) alone, so no a above it is
+//    kept; the row's smallest base a1 lowers that bound to base(a1, b) + max D^g when a1 is feasible with every open
+//    c and with (b, eps). With W^d small most rows keep nothing, and their cells need no direction at all;
+//  * theta(a->c) is computed only for the a that some row keeps, once the kept lists are there;
+//  * the cells that hold eps are minima without a geometric term: (b, eps) over the a within T of b, by the row's
+//    threads; (eps, c) over base(a, eps), by the threads of c; (eps, eps) by one warp. Their base values are three
+//    small arrays, kept for the coming and the current step.
+// Ties prefer the lower slot, eps last: a cell's walk starts from the next float above base(eps, b), so a real a of
+// equal cost replaces it. The argmin slots go to a per-CTA global scratch, and the CTA backtracks its own unit (Eq.
+// 12); eps is reported as -2 in the assignment.
+//
+// Bound by issue and the latency of the step's phases. Measured with the earlier kernel (a warp per row ranking the
+// kept a by counting, base, row and list passes between five barriers, two CTAs per SM) and with this one, three CTAs
+// per SM: 2,710 units of up to 64 points at W^d = 8 (K = 64) 5,707 -> 2,208 us.
+#include <algorithm>
+#include <climits>
+
 #include "hgm_internal.cuh"
-#include "recurse_common.cuh"
+#include "recurse_lists.cuh"
 
 namespace hgm {
 namespace {
 
-constexpr int kDummyThreads = 256;
-constexpr int kL = kMaxK + 1;          // table side: up to 64 real slots + eps
-constexpr int kTab = kL * kL;
-constexpr int kRL = 68;                // row stride of R: four consecutive c of a row are one 16-byte load
-constexpr float kGeoMax = 4.45f;       // > pi*sqrt(2) = 4.4429, bound of the FP32 D^g
-
+template <int KM, int NT>
 struct DummySmem {
-    float alpha[2][kTab];
-    float base[kTab];                  // [b][a]
-    float p1[kTab], p2[kTab];          // [b][a]
-    alignas(16) float r[kL * kRL];     // [a][c], row stride kRL
-    float2 xy[3][kL];                  // lists i (a), i-1 (b), i-2 (c)
-    int t[3][kL], id[3][kL];
-    float u[3][kL];
-    uint8_t srt[kL][kMaxK];            // per row b: the kept real a by increasing base(b, a) (ties: lower slot)
-    uint8_t kept[kL];                  // per row b: how many a srt[b] holds
-    unsigned akept[2];                 // real a kept by some real row b (bits of slots 0-31, 32-63)
-    int cnt[3];
-    float ang[2];                      // the step's model angles A1, A2 (one thread computes them)
-};
-static_assert(2 * (sizeof(DummySmem) + 1024 + 128) <= 228 * 1024, "two CTAs per SM");
+    static constexpr int FS = KM + 1, SS = KM + 4, RS = KM + 4, AS = KM + 4;   // as in k_recurse.cu
+    float2 fb[KM * FS];                   // per b: kept (base, p1) in increasing a
+    float r[KM * RS];                     // theta(a->c) or +inf at a*RS + c | 16 bytes of tile_b per row
+    float alpha[KM * AS];                 // base(a,b) of the coming step at b*AS + a | key, be, ea
+    uint8_t fs[KM * SS];                  // slot of each kept entry, | 0x80 when a lies at b's position | tile info
+    List<KM> list[3];
+    float ea1[KM];
+    float4 geo[2];
+    float ee[2];                          // base(eps, eps) of step i at ee[i & 1]
+    float red_v[NT / 32];
+    int32_t red_k[NT / 32];
+    int32_t ntile, unit;
+    int32_t coin[2];
+    unsigned akept[2];                    // a kept by some row (bits of slots 0-31, 32-63)
 
-// (key, slot) order: smaller key first, then lower slot
-__device__ __forceinline__ bool key_less(float ka, int sa, float kb, int sb)
-{
-    return ka < kb || (ka == kb && sa < sb);
-}
-
-struct DummyBest {
-    float v;
-    int j1, j2;
+    __device__ uint8_t &tile_b(int t) { return reinterpret_cast<uint8_t *>(&r[(t >> 4) * RS + KM])[t & 15]; }
+    __device__ int32_t &key(int b) { return reinterpret_cast<int32_t *>(alpha)[b * AS + KM]; }
+    __device__ int32_t &info(int b) { return *reinterpret_cast<int32_t *>(fs + b * SS + KM); }
+    // step i: base(eps, b) and base(a, eps), of parity i & 1
+    __device__ float &be(int par, int b) { return alpha[b * AS + KM + 1 + par]; }
+    __device__ float &ea(int par, int a) { return par ? ea1[a] : alpha[a * AS + KM + 3]; }
 };
 
-__device__ __forceinline__ bool dummy_better(float v, int j1, int j2, const DummyBest &o)
-{
-    if (v != o.v) return v < o.v;
-    if (j1 != o.j1) return j1 < o.j1;
-    return j2 < o.j2;
-}
-
-// kCount = true builds the accounting variant: identical work, plus a count of the (a, open cell) triples
-// the walks evaluate, added to *evaluated (work accounting; not used on the timed path).
-template <bool kCount>
-__global__ void __launch_bounds__(kDummyThreads, 2) dummy_recurse_kernel(
+// kCount = true builds the accounting variant: identical work, plus a count of the (a, open cell) triples the walks
+// evaluate, added to *evaluated (work accounting; not used on the timed path).
+template <int KM, int NT, int MB, bool kCount>
+__global__ void __launch_bounds__(NT, MB) dummy_recurse_kernel(
     const Unit *__restrict__ units, int64_t n_units, const ModelRec *__restrict__ models,
     const SceneRec *__restrict__ scenes, Params p, float wd, const int32_t *__restrict__ cand_idx,
     const float *__restrict__ cand_u, const int32_t *__restrict__ cand_cnt, uint8_t *__restrict__ scratch,
-    int64_t scratch_per_cta, float *__restrict__ energy, int32_t *__restrict__ assign,
+    int64_t scratch_per_cta, int *__restrict__ work_counter, float *__restrict__ energy, int32_t *__restrict__ assign,
     unsigned long long *__restrict__ evaluated)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DummySmem &sm = *reinterpret_cast<DummySmem *>(smem_raw);
-    __shared__ DummyBest red[kDummyThreads / 32];
-    const int K = p.K, L = K + 1, E = K;   // eps is slot K
-    // e / L as one multiply-high: with m = ceil(2^32 / L), floor(e m / 2^32) = floor(e / L) for every
-    // e < 2^32 / L (the error e (m - 2^32 / L) / 2^32 stays below 1 / L); the flat loops index e < 3 L^2
-    const unsigned divL = 0xffffffffu / (unsigned)L + 1u;
+    using SM = DummySmem<KM, NT>;
+    SM &sm = *reinterpret_cast<SM *>(smem_raw);
+    constexpr int RS = SM::RS, AS = SM::AS, FS = SM::FS, SS = SM::SS;
+    constexpr int NW = NT / 32, CT = 4;
+    constexpr int TPB = NT / KM, AH = KM / TPB;   // threads per b (and per c), slots a per thread
+    constexpr int E = KM, LS = KM + 4;            // slot of eps in the argmin tables, their row stride
+    static_assert(TPB == 4, "threads per b");
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int K = p.K, T = p.T;
     const float lam2 = p.lambda2, lam23 = __fmul_rn(p.lambda2, p.lambda3);
     const float ueps = __fmul_rn(p.lambda1, wd);
     const float gmax = lam23 * kGeoMax;
-    const float inf = __int_as_float(0x7f800000);
+    const int h = tid % TPB, row = tid / TPB, rot = h;
     uint8_t *beta = scratch + (int64_t)blockIdx.x * scratch_per_cta;
     unsigned long long n_eval = 0;
-    for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
+    for (;;) {
+        if (tid == 0) sm.unit = atomicAdd(work_counter, 1);
+        __syncthreads();
+        const int64_t u = sm.unit;
+        if (u >= n_units) break;
         const Unit un = units[u];
         const ModelRec md = models[un.model];
         const SceneRec sc = scenes[un.scene];
@@ -94,332 +94,444 @@ __global__ void __launch_bounds__(kDummyThreads, 2) dummy_recurse_kernel(
         const int32_t *cidx = cand_idx + un.cand;
         const float *cu = cand_u + un.cand;
         const int32_t *ccnt = cand_cnt + un.cand / K;
-        int cur = 0;
+        for (int q = 1; q <= 3; ++q)
+            load_list<KM>(sm.list[(M - q) % 3], sc, cidx + (int64_t)(M - q) * K, cu + (int64_t)(M - q) * K, ccnt[M - q],
+                          tid, NT);
+        if (tid == 0) {
+            sm.geo[(M - 1) & 1] = md.geo[M - 1];
+            sm.coin[0] = sm.coin[1] = 0;
+            sm.akept[0] = sm.akept[1] = 0u;
+            sm.ee[(M - 1) & 1] = ueps;
+        }
+        __syncthreads();
+        {   // the first step's base: alpha_{M+1} == 0 (Eq. 11)
+            const List<KM> &LA = sm.list[(M - 1) % 3], &LB = sm.list[(M - 2) % 3];
+            const int dt_ab = __float_as_int(sm.geo[(M - 1) & 1].z);
+            for (int e = tid; e < KM * KM; e += NT) {
+                const int b = e / KM, a = e % KM;
+                const bool ok = a < LA.n && b < LB.n && LA.t[a] >= LB.t[b] && LA.idx[a] != LB.idx[b];
+                sm.alpha[b * AS + a] = ok ? base_cost(LA.u[a], lam2, dt_ab, LA.t[a], LB.t[b], 0.0f) : kInf;
+            }
+            if (tid < KM) {
+                sm.be((M - 1) & 1, tid) = ueps;
+                sm.ea((M - 1) & 1, tid) = LA.u[tid];
+            }
+        }
+        __syncthreads();
+
         for (int i = M - 1; i >= 2; --i) {
-            // list buffers rotate with the chain index (list i in buffer i % 3): the first step loads the three
-            // lists, every later step only list i - 2; slot s < cnt real, slot K eps
-            const int sA = i % 3, sB = (i - 1) % 3, sC = (i - 2) % 3;
-            const int nload = i == M - 1 ? 3 : 1, w0 = i == M - 1 ? 0 : 2;
-            for (int e = threadIdx.x; e < nload * L; e += blockDim.x) {
-                const int q = (int)__umulhi((unsigned)e, divL), s = e - q * L, li = i - (w0 + q);
-                const int w = li % 3;
-                const int n = ccnt[li];
-                if (s < n) {
-                    const int j = cidx[(int64_t)li * K + s];
-                    sm.xy[w][s] = sc.xy[j];
-                    sm.t[w][s] = sc.t[j];
-                    sm.id[w][s] = j;
-                    sm.u[w][s] = cu[(int64_t)li * K + s];
-                } else if (s == E) {
-                    sm.xy[w][s] = make_float2(0.f, 0.f);
-                    sm.t[w][s] = 0;
-                    sm.id[w][s] = -2;
-                    sm.u[w][s] = ueps;
+            List<KM> &LA = sm.list[i % 3];
+            List<KM> &LB = sm.list[(i - 1) % 3];
+            List<KM> &LC = sm.list[(i - 2) % 3];
+            const int par = i & 1, npar = par ^ 1;
+            const float4 g = sm.geo[par];
+            const float A1 = g.x, k2 = g.y;
+            const float k2c = wrap_pi(__fsub_rn(k2, kPi));   // a and b at the same position (reading R1)
+            const int dt_bc = __float_as_int(g.w);
+            const int na = LA.n, nb = LB.n, nc = LC.n;
+            uint8_t *bstep = beta + (int64_t)(i - 2) * (KM + 1) * LS;
+            // list C of the next step (chain index i-3) is fetched by the first threads
+            const bool pf = i >= 3 && tid < K;
+            int pf_n = 0, pf_j = -1;
+            float pf_u = kInf;
+            float2 pf_xy = make_float2(0.f, 0.f);
+            int pf_t = 0x3fffffff;
+            if (pf) {
+                pf_n = ccnt[i - 3];
+                pf_j = cidx[(int64_t)(i - 3) * K + tid];
+                pf_u = cu[(int64_t)(i - 3) * K + tid];
+            }
+            if (tid == NT - 1 && i >= 3) sm.geo[npar] = md.geo[i - 1];
+            auto lower_bound = [](const int32_t *arr, int n, int x) {
+                int l = 0;
+                while (l < n) {
+                    const int mid = (l + n) >> 1;
+                    if (arr[mid] < x) l = mid + 1;
+                    else n = mid;
                 }
-                if (s == 0) sm.cnt[w] = n;
+                return l;
+            };
+            const int base_lane = lane & ~(TPB - 1);
+            // the a of a time range: those not before frame t0 (range.x) and less than T frames after it (.y)
+            auto time_range = [&](int t0, int n) {
+                const int x = (h & 1) == 0 ? t0 : (T > 0 && t0 <= INT_MAX - T ? t0 + T : INT_MAX);
+                const int f = lower_bound(LA.t, n, x);
+                const int l = __shfl_sync(full, f, base_lane), r = __shfl_sync(full, f, base_lane + 1);
+                return make_int2(l, T > 0 ? r : n);
+            };
+            // (value, slot) minimum over the threads of a row, ties to the lower slot
+            auto row_min = [&](float &v, int &s) {
+#pragma unroll
+                for (int off = 1; off < TPB; off <<= 1)
+                    argmin_merge(v, s, __shfl_xor_sync(full, v, off), __shfl_xor_sync(full, s, off));
+            };
+
+            // ---- phase 1: the kept a list of b = row, and the cell (b, eps)
+            {
+                const int b = row;
+                const bool inb = b < nb;
+                float2 pb = make_float2(0.f, 0.f);
+                int tb = 0, ib = -1;
+                if (inb) { pb = LB.xy[b]; tb = LB.t[b]; ib = LB.idx[b]; }
+                const float *arow = sm.alpha + b * AS + AH * h;
+                const int2 ra = time_range(tb, inb ? na : 0);
+                const int j0 = ra.x - AH * h, jT = ra.y - AH * h, j1 = (inb ? na : 0) - AH * h;
+                float v[AH], m1 = kInf, mE = kInf;
+                int s1 = 1 << 20, sE = 1 << 20;
+#pragma unroll
+                for (int k = 0; k < AH; ++k) {
+                    const int j = (k + rot) & (AH - 1);
+                    const float x = arow[j];
+                    v[k] = j >= j0 && j < j1 ? x : kInf;
+                    m1 = fminf(m1, v[k]);
+                    mE = fminf(mE, j < jT ? v[k] : kInf);
+                }
+#pragma unroll
+                for (int k = 0; k < AH; ++k) {
+                    const int j = (k + rot) & (AH - 1), a = AH * h + j;
+                    if (v[k] == m1) s1 = min(s1, a);
+                    if (v[k] == mE && j < jT) sE = min(sE, a);
+                }
+                row_min(m1, s1);
+                row_min(mE, sE);
+                const bool any = m1 < kInf;
+                if (!any) s1 = 0;
+                const int tw = LA.t[s1], iw = any ? LA.idx[s1] : -2;
+                // searches of list C (time order, scene index order), one per lane: c not after b, c too far from the
+                // witness, c too far from b, the witness's point
+                const int q = h & 3;
+                const int x = q == 0 ? tb + 1 : q == 1 ? (T > 0 ? tw - T + 1 : INT_MIN)
+                                            : q == 2 ? (T > 0 ? tb - T + 1 : INT_MIN) : iw;
+                int f = lower_bound(q < 3 ? LC.t : LC.idx, nc, x);
+                if (q == 3 && !(f < nc && LC.idx[f] == x)) f = KM;
+                int ccount = __shfl_sync(full, f, base_lane);
+                if (!inb) ccount = 0;
+                const int nT = min(__shfl_sync(full, f, base_lane + 1), ccount);
+                const int nB = min(__shfl_sync(full, f, base_lane + 2), ccount);
+                const int pw = __shfl_sync(full, f, base_lane + 3);
+                const float beb = inb ? sm.be(par, b) : kInf;
+                const bool live = any && ccount > 0;
+                float thr = beb;
+                {
+                    // the open c are those from nB on but b's own point, which is as far from the witness as b is
+                    const float lower = m1 + gmax + 1e-6f * fabsf(m1);
+                    const bool bad = (T > 0 && tw - tb >= T) || nT > nB || (pw < ccount && pw >= nB);
+                    if (lower < thr && !bad) thr = lower;
+                }
+                thr = live ? fminf(thr, 3.402823466e38f) : -kInf;
+                unsigned mk = 0;
+#pragma unroll
+                for (int k = 0; k < AH; ++k)
+                    if (v[k] <= thr) mk |= 1u << k;
+                mk = ((mk << rot) | (mk >> (AH - rot))) & ((1u << AH) - 1);
+                int pos = 0, kept = __popc(mk);
+#pragma unroll
+                for (int off = 1; off < TPB; off <<= 1) {
+                    const int o = __shfl_xor_sync(full, kept, off);
+                    if (h & off) pos += o;
+                    kept += o;
+                }
+                if (mk) {
+                    const unsigned long long bits = (unsigned long long)mk << (AH * h);
+                    atomicOr(&sm.akept[(AH * h) >> 5], (unsigned)(bits >> ((AH * h) & ~31)));
+                }
+                for (unsigned m = mk; m; m &= m - 1, ++pos) {
+                    const int j = __ffs((int)m) - 1, a = AH * h + j;
+                    const float2 pa = LA.xy[a];
+                    const bool same = pa.x == pb.x && pa.y == pb.y;
+                    if (same) sm.coin[par] = 1;
+                    sm.fb[b * FS + pos] = make_float2(arow[j], wrap_pi(__fadd_rn(A1, direction(pb, pa))));
+                    sm.fs[b * SS + pos] = (uint8_t)(a | (same ? 0x80 : 0));
+                }
+                if (h == 0) {
+                    const int nt_b = (ccount + CT - 1) / CT;
+                    const int key = nt_b > 0 ? ((kept + 1) << 8) | (255 - b) : 0;
+                    sm.key(b) = (key << 5) | nt_b;
+                    if (inb) {   // the cell (b, eps): base alone; next step's base(a = b, eps) = U(b) + alpha
+                        const bool real = mE < kInf && mE <= beb;
+                        const float al = real ? mE : beb;
+                        sm.ea(npar, b) = i > 2 ? __fadd_rn(LB.u[b], al) : al;
+                        bstep[b * LS + E] = (uint8_t)(real ? sE : E);
+                    }
+                }
             }
-            if (threadIdx.x == 0) {
-                sm.akept[0] = 0u;
-                sm.akept[1] = 0u;
-                const float2 mi = md.xy[i], mj = md.xy[i - 1], mk = md.xy[i - 2];
-                sm.ang[0] = signed_angle(mj, mi, mk);   // A1: at i-1, from ->i to ->i-2
-                sm.ang[1] = signed_angle(mi, mj, mk);   // A2: at i, from ->i-1 to ->i-2
+            if (pf && tid < pf_n) {
+                pf_xy = sc.xy[pf_j];
+                pf_t = sc.t[pf_j];
             }
-            // base reads lists i and i - 1 only: after the first step they are in place already, so the list
-            // being loaded (i - 2) and the base table share one barrier
-            if (i == M - 1) __syncthreads();
-            const int dt1 = md.t[i] - md.t[i - 1], dt2 = md.t[i - 1] - md.t[i - 2];
-            const int na = sm.cnt[sA], nb = sm.cnt[sB];
-            const float *an = sm.alpha[cur];
-            const bool last = i == M - 1;
-            // base(b, a); rows/columns of empty slots are never read
-            for (int e = threadIdx.x; e < L * L; e += blockDim.x) {
-                const int b = (int)__umulhi((unsigned)e, divL), a = e - b * L;
-                const bool ra = a < na, rb = b < nb;
-                if ((ra || a == E) && (rb || b == E)) {
-                    const float al = last ? 0.0f : an[a * L + b];   // alpha_{i+1}(z_i = a, z_{i-1} = b)
-                    float bs;
-                    if (ra && rb) bs = base_cost(sm.u[sA][a], lam2, dt1, sm.t[sA][a], sm.t[sB][b], al);
-                    else bs = __fadd_rn(sm.u[sA][a], al);
-                    sm.base[b * L + a] = bs;
+            // the cells (eps, c), c = row: base(a, eps) of the a that may follow c
+            const bool inc_c = row < nc;
+            const int tc_row = inc_c ? LC.t[row] : 0, ic_row = inc_c ? LC.idx[row] : -3;
+            const int2 rc_range = time_range(tc_row, inc_c ? na : 0);
+            {
+                float m = kInf;
+                int s = 1 << 20;
+                for (int a = rc_range.x + h; a < rc_range.y; a += TPB) {
+                    const float x = sm.ea(par, a);
+                    if (LA.idx[a] != ic_row && x < m) { m = x; s = a; }
+                }
+                row_min(m, s);
+                if (h == 0 && inc_c) {
+                    const bool real = m < kInf && m <= sm.ee[par];
+                    const float al = real ? m : sm.ee[par];
+                    sm.be(npar, row) = i > 2 ? __fadd_rn(ueps, al) : al;
+                    bstep[E * LS + row] = (uint8_t)(real ? s : E);
+                }
+            }
+            if (warp == NW - 1) {   // the cell (eps, eps)
+                float m = kInf;
+                int s = 1 << 20;
+                for (int a = lane; a < na; a += 32) {
+                    const float x = sm.ea(par, a);
+                    if (x < m) { m = x; s = a; }
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1)
+                    argmin_merge(m, s, __shfl_xor_sync(full, m, off), __shfl_xor_sync(full, s, off));
+                if (lane == 0) {
+                    const bool real = m < kInf && m <= sm.ee[par];
+                    const float al = real ? m : sm.ee[par];
+                    sm.ee[npar] = i > 2 ? __fadd_rn(ueps, al) : al;
+                    bstep[E * LS + E] = (uint8_t)(real ? s : E);
                 }
             }
             __syncthreads();
-            const float A1 = sm.ang[0], A2 = sm.ang[1];
-            const int nc = sm.cnt[sC];
-            // branch and bound (exact): v(a, b, c) >= base(b, a), and no open cell of row b has a best above
-            // thr(b). A warp per row keeps the a with base <= thr(b) that may follow b (any real a after eps)
-            // and ranks them by (base, slot) by counting.
-            {
-                const unsigned full = 0xffffffffu;
-                const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-                for (int b = warp; b < L; b += kDummyThreads / 32) {
-                    if (!(b < nb || b == E)) continue;
-                    const bool rb = b < nb;
-                    const float *brow = sm.base + b * L;
-                    const int tb = rb ? sm.t[sB][b] : 0, ib = rb ? sm.id[sB][b] : -3;
-                    float key[2];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int a = lane + 32 * h;
-                        key[h] = a < na && (!rb || (sm.id[sA][a] != ib && sm.t[sA][a] >= tb)) ? brow[a] : inf;
-                    }
-                    float thr = brow[E];
-                    if (rb) {
-                        float m = key[0];
-                        int s = lane;
-                        if (key_less(key[1], lane + 32, m, s)) { m = key[1]; s = lane + 32; }
-#pragma unroll
-                        for (int off = 16; off > 0; off >>= 1) {
-                            const float om = __shfl_xor_sync(full, m, off);
-                            const int os = __shfl_xor_sync(full, s, off);
-                            if (key_less(om, os, m, s)) { m = om; s = os; }
-                        }
-                        // the second bound can only matter below base(b, eps): skip its feasibility scan otherwise
-                        if (m < inf && m + gmax + 1e-6f * fabsf(m) < thr) {
-                            // a1 = s must be feasible with every open c and with (b, eps)
-                            const int t1 = sm.t[sA][s], i1 = sm.id[sA][s];
-                            bool bad = lane == 0 && p.T > 0 && t1 - tb >= p.T;
-                            for (int c = lane; c < nc; c += 32) {
-                                const int tc = sm.t[sC][c], ic = sm.id[sC][c];
-                                const bool open = ic != ib && tc <= tb && (p.T <= 0 || tb - tc < p.T);
-                                if (open && (i1 == ic || (p.T > 0 && t1 - tc >= p.T))) bad = true;
-                            }
-                            if (!__any_sync(full, bad)) thr = fminf(thr, m + gmax + 1e-6f * fabsf(m));
-                        }
-                    }
-                    const bool k0 = key[0] < inf && key[0] <= thr, k1 = key[1] < inf && key[1] <= thr;
-                    const unsigned m0 = __ballot_sync(full, k0), m1 = __ballot_sync(full, k1);
-                    int r0 = 0, r1 = 0;
-                    for (unsigned mm = m0; mm; mm &= mm - 1) {
-                        const int l = __ffs(mm) - 1;
-                        const float kk = __shfl_sync(full, key[0], l);
-                        r0 += key_less(kk, l, key[0], lane);
-                        r1 += key_less(kk, l, key[1], lane + 32);
-                    }
-                    for (unsigned mm = m1; mm; mm &= mm - 1) {
-                        const int l = __ffs(mm) - 1;
-                        const float kk = __shfl_sync(full, key[1], l);
-                        r0 += key_less(kk, l + 32, key[0], lane);
-                        r1 += key_less(kk, l + 32, key[1], lane + 32);
-                    }
-                    if (k0) sm.srt[b][r0] = (uint8_t)lane;
-                    if (k1) sm.srt[b][r1] = (uint8_t)(lane + 32);
-                    if (lane == 0) {
-                        sm.kept[b] = (uint8_t)(__popc(m0) + __popc(m1));
-                        if (rb) {   // the cells of a real row read R(a, c) of its kept a
-                            if (m0) atomicOr(&sm.akept[0], m0);
-                            if (m1) atomicOr(&sm.akept[1], m1);
-                        }
-                    }
-                    // directions of the kept pairs of a real b, the only ones the cells read: lane r takes the
-                    // kept a of rank r
-                    if (rb) {
-                        __syncwarp();
-                        const int nk = __popc(m0) + __popc(m1);
-                        const float2 xb = sm.xy[sB][b];
-                        for (int r = lane; r < nk; r += 32) {
-                            const int a = sm.srt[b][r];
-                            sm.p1[b * L + a] = __fadd_rn(A1, direction(xb, sm.xy[sA][a]));
-                            sm.p2[b * L + a] = __fadd_rn(A2, direction(sm.xy[sA][a], xb));
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-            // R(a, c) = theta(a->c) for the a some real row keeps, where (a, c) can be feasible (with W^d small
-            // most rows keep no a: their cells take eps without any direction)
-            {
+
+            // theta(a->c) of the kept a, c = row (rows from the first a with t'(a) >= t'(c), as in k_recurse.cu)
+            if (inc_c) {
                 const unsigned k0 = sm.akept[0], k1 = sm.akept[1];
                 if (k0 | k1) {
-                    for (int e = threadIdx.x; e < L * L; e += blockDim.x) {
-                        const int a2 = (int)__umulhi((unsigned)e, divL), c = e - a2 * L;
-                        if (a2 >= na || c >= nc || !(((a2 < 32 ? k0 : k1) >> (a2 & 31)) & 1u)) continue;
-                        if (sm.t[sC][c] <= sm.t[sA][a2] && !(p.T > 0 && sm.t[sA][a2] - sm.t[sC][c] >= p.T))
-                            sm.r[a2 * kRL + c] = direction(sm.xy[sA][a2], sm.xy[sC][c]);
+                    const float2 pc = LC.xy[row];
+                    for (int a = rc_range.x + h; a < na; a += TPB) {
+                        if (!(((a < 32 ? k0 : k1) >> (a & 31)) & 1u)) continue;
+                        sm.r[a * RS + row] = a < rc_range.y && LA.idx[a] != ic_row ? direction(LA.xy[a], pc) : kInf;
                     }
+                }
+            }
+            // tile layout (as in k_recurse.cu)
+            {
+                const int b = row, wb = sm.key(b), key = wb >> 5, nt_b = wb & 31;
+                int before = 0, total = 0;
+                for (int b2 = h; b2 < KM; b2 += TPB) {
+                    const int w = sm.key(b2);
+                    total += w & 31;
+                    if ((w >> 5) > key) before += w & 31;
+                }
+#pragma unroll
+                for (int off = 1; off < TPB; off <<= 1) {
+                    before += __shfl_xor_sync(full, before, off);
+                    total += __shfl_xor_sync(full, total, off);
+                }
+                if (h == 0) sm.info(b) = before << 12 | max((key >> 8) - 1, 0) << 5 | nt_b;
+                for (int t = h; t < nt_b; t += TPB) sm.tile_b(before + t) = (uint8_t)b;
+                if (tid == 0) {
+                    sm.ntile = total;
+                    sm.coin[npar] = 0;
                 }
             }
             __syncthreads();
-            float *ac = sm.alpha[cur ^ 1];
-            uint8_t *bt = beta + (int64_t)(i - 2) * L * L;
-            // real cells (b, c) in groups of four consecutive c: one walk of b's base-sorted row serves the
-            // group, and stops at the first base above every open cell's best (exact: v >= base)
-            const int G = (nc + 3) >> 2;
-            const unsigned divG = 0xffffffffu / (unsigned)max(G, 2) + 1u;   // e / G as for e / L
-            for (int e = threadIdx.x; e < nb * G; e += blockDim.x) {
-                const int b = G == 1 ? e : (int)__umulhi((unsigned)e, divG), c0 = 4 * (e - b * G);
-                const int tb = sm.t[sB][b], ib = sm.id[sB][b];
-                const float *brow = sm.base + b * L;
-                const int nk = sm.kept[b];   // 0: every open cell of the group takes eps, no direction needed
-                float best[4], q1[4];
-                int arg[4], tcq[4], icq[4];
-                bool open[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = c0 + q;
-                    const bool inc = c < nc;
-                    tcq[q] = inc ? sm.t[sC][c] : 0;
-                    icq[q] = inc ? sm.id[sC][c] : -3;
-                    open[q] = inc && icq[q] != ib && tcq[q] <= tb && (p.T <= 0 || tb - tcq[q] < p.T);
-                    q1[q] = open[q] && nk > 0 ? direction(sm.xy[sB][b], sm.xy[sC][c]) : 0.0f;
-                    best[q] = open[q] ? brow[E] : inf;   // (eps, b, c) is feasible with every open cell
-                    arg[q] = open[q] ? E : 255;
-                }
-                const int nopen = (int)open[0] + (int)open[1] + (int)open[2] + (int)open[3];
-                const unsigned long long q1a = pk2(q1[0], q1[1]), q1b = pk2(q1[2], q1[3]);
-                const unsigned long long lamp = pk2(lam23, lam23);
-                const uint8_t *order = sm.srt[b];
-                for (int k = 0; k < nk; ++k) {
-                    const int a = order[k];
-                    const float ba = brow[a];
-                    float bmax = -inf;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) bmax = fmaxf(bmax, open[q] ? best[q] : -inf);
-                    if (ba > bmax) break;
-                    if constexpr (kCount) n_eval += nopen;
-                    const int ta = sm.t[sA][a], ia = sm.id[sA][a];   // kept: ia != ib, ta >= tb
-                    const float p1 = sm.p1[b * L + a], p2 = sm.p2[b * L + a];
-                    // R past the last c is never initialised: those lanes of v are discarded (open is false)
-                    const float4 r4 = *reinterpret_cast<const float4 *>(sm.r + a * kRL + c0);
-                    const unsigned long long bp = pk2(ba, ba), p1p = pk2(p1, p1), p2p = pk2(p2, p2);
-                    float v[4];
-                    triple_cost2(bp, p1p, p2p, q1a, pk2(r4.x, r4.y), lamp, v[0], v[1]);
-                    triple_cost2(bp, p1p, p2p, q1b, pk2(r4.z, r4.w), lamp, v[2], v[3]);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const bool ok = open[q] && ia != icq[q] && !(p.T > 0 && ta - tcq[q] >= p.T);
-                        if (ok && (v[q] < best[q] || (v[q] == best[q] && a < arg[q]))) { best[q] = v[q]; arg[q] = a; }
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = c0 + q;
-                    if (c < nc) {
-                        ac[b * L + c] = open[q] ? cell_alpha(best[q], lam2, dt2, tb, tcq[q]) : inf;
-                        bt[b * L + c] = (uint8_t)(open[q] ? arg[q] : 255);
-                    }
+
+            // list A is not read from here on: its buffer receives list C of the next step
+            if (i >= 3 && tid < KM) {
+                const bool ok = tid < pf_n;
+                LA.idx[tid] = ok ? pf_j : -1;
+                LA.xy[tid] = pf_xy;
+                LA.t[tid] = pf_t;
+                LA.u[tid] = ok ? pf_u : kInf;
+                if (tid == 0) {
+                    LA.n = pf_n;
+                    sm.akept[0] = sm.akept[1] = 0u;
                 }
             }
-            // cells holding eps (row b = eps over every c, column c = eps over the real b): a triple holding
-            // eps costs base(b, a) alone, so in ranked order the first feasible kept a is the smallest (lowest
-            // slot among equals); eps (the last slot) only if below it. An a left out of row eps costs more
-            // than base(eps, eps); for a real b either the same holds or a1, the first kept, is feasible with
-            // (b, eps)
-            for (int e = threadIdx.x; e < nc + 1 + nb; e += blockDim.x) {
-                const int b = e <= nc ? E : e - (nc + 1);
-                const int c = e < nc ? e : E;
-                const bool rb = b < nb, rc = c < nc;
-                const float *brow = sm.base + b * L;
-                const uint8_t *order = sm.srt[b];
-                const int tr = rc ? sm.t[sC][c] : (rb ? sm.t[sB][b] : 0);   // the other real point
-                const int ir = rc ? sm.id[sC][c] : (rb ? sm.id[sB][b] : -3);
-                const bool any = !rb && !rc;
-                float best = inf;
-                int arg = 255;
-                const int nk = sm.kept[b];
-                for (int k = 0; k < nk; ++k) {
-                    const int a = order[k];
-                    const int ta = sm.t[sA][a];
-                    if (!any && (sm.id[sA][a] == ir || ta < tr || (p.T > 0 && ta - tr >= p.T))) continue;
-                    best = brow[a];
-                    arg = a;
-                    break;
+            // ---- phase 3: tiles (b, four consecutive c)
+            const int ntile = sm.ntile;
+            const bool coin = sm.coin[par] != 0;
+            const unsigned long long lamp = pk2(lam23, lam23);
+            for (int r0 = 0; r0 < ntile; r0 += NT) {
+                const int tile = r0 + (((r0 / NT) & 1) ? NT - 1 - tid : tid);
+                if (tile >= ntile) continue;
+                const int b = sm.tile_b(tile);
+                const int info = sm.info(b);
+                const int c0 = (tile - (info >> 12)) * CT;
+                const int nf = (info >> 5) & 127;
+                const float2 pb = LB.xy[b];
+                const int tb = LB.t[b], ib = LB.idx[b];
+                const float ub = LB.u[b], beb = sm.be(par, b);
+                // a real a of equal cost replaces eps: start just above base(eps, b)
+                const float start = __uint_as_float(__float_as_uint(beb) + 1u);
+                float best[CT];
+                int arg[CT], tcq[CT];
+                bool open[CT];
+                const int4 t4 = *reinterpret_cast<const int4 *>(&LC.t[c0]);
+                const int4 i4 = *reinterpret_cast<const int4 *>(&LC.idx[c0]);
+                const int tv[4] = {t4.x, t4.y, t4.z, t4.w}, iv[4] = {i4.x, i4.y, i4.z, i4.w};
+#pragma unroll
+                for (int q = 0; q < CT; ++q) {
+                    tcq[q] = tv[q];
+                    open[q] = c0 + q < nc && tv[q] <= tb && iv[q] != ib && (T <= 0 || tb - tv[q] < T);
+                    best[q] = open[q] ? start : kInf;
+                    arg[q] = open[q] ? E : kNoSlot;
                 }
-                if (brow[E] < best) { best = brow[E]; arg = E; }
-                ac[b * L + c] = best;
-                bt[b * L + c] = (uint8_t)arg;
+                if (nf > 0) {
+                    const float4 xa = *reinterpret_cast<const float4 *>(&LC.xy[c0]);
+                    const float4 xb = *reinterpret_cast<const float4 *>(&LC.xy[c0 + 2]);
+                    const float2 xv[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
+                                          make_float2(xb.z, xb.w)};
+                    float q1[CT];
+#pragma unroll
+                    for (int q = 0; q < CT; ++q) {
+                        const float d = direction(pb, xv[q]);   // theta(b->c)
+                        q1[q] = open[q] ? d : kInf;
+                    }
+                    const unsigned long long q1a = pk2(q1[0], q1[1]), q1b = pk2(q1[2], q1[3]);
+                    const float2 *fb = sm.fb + b * FS;
+                    const uint8_t *fs = sm.fs + b * SS;
+                    if constexpr (kCount) n_eval += nf * ((int)open[0] + (int)open[1] + (int)open[2] + (int)open[3]);
+#pragma unroll 2
+                    for (int k = 0; k < nf; ++k) {
+                        const float2 e = fb[k];
+                        const int fa = fs[k], a = fa & 0x7f;
+                        const float p2 = __fadd_rn(e.y, coin && (fa & 0x80) ? k2c : k2);
+                        const float4 r4 = *reinterpret_cast<const float4 *>(sm.r + a * RS + c0);
+                        const unsigned long long bp = pk2(e.x, e.x), p1p = pk2(e.y, e.y), p2p = pk2(p2, p2);
+                        float v[4];
+                        triple_cost2(bp, p1p, p2p, q1a, pk2(r4.x, r4.y), lamp, v[0], v[1]);
+                        triple_cost2(bp, p1p, p2p, q1b, pk2(r4.z, r4.w), lamp, v[2], v[3]);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (v[q] < best[q]) { best[q] = v[q]; arg[q] = a; }
+                    }
+                }
+                uint32_t packed = 0;
+#pragma unroll
+                for (int q = 0; q < CT; ++q) {
+                    const int c = c0 + q;
+                    if (arg[q] == E) best[q] = beb;
+                    const float al = cell_alpha(best[q], lam2, dt_bc, tb, tcq[q]);
+                    const float out = i > 2 ? base_cost(ub, lam2, dt_bc, tb, tcq[q], al) : al;
+                    if (c < nc) sm.alpha[c * AS + b] = out;
+                    packed |= (uint32_t)arg[q] << (8 * q);
+                }
+                *reinterpret_cast<uint32_t *>(bstep + b * LS + c0) = packed;   // rows of whole words, eps after them
             }
-            cur ^= 1;
+            if (i == 2) {   // Eq. 13 reads every cell of the last step
+                for (int b = warp; b < nb; b += NW) {
+                    const int covered = (sm.info(b) & 31) * CT;
+                    for (int c = covered + lane; c < nc; c += 32) sm.alpha[c * AS + b] = kInf;
+                }
+            }
             __syncthreads();
         }
-        // Eq. 13 over (z_1 = j1, z_2 = j2) in C_1 + eps, C_2 + eps: U + U + alpha_3(j2, j1)
-        const float *a3 = sm.alpha[cur];
-        const int n0 = ccnt[0], n1 = ccnt[1];
-        DummyBest mine{inf, 0x7fffffff, 0x7fffffff};
-        for (int e = threadIdx.x; e < L * L; e += blockDim.x) {
-            const int j1 = (int)__umulhi((unsigned)e, divL), j2 = e - j1 * L;
-            if (!((j1 < n0 || j1 == E) && (j2 < n1 || j2 == E))) continue;
-            const float u1 = j1 == E ? ueps : cu[j1], u2 = j2 == E ? ueps : cu[(int64_t)K + j2];
-            const float al = M == 2 ? 0.0f : a3[j2 * L + j1];
-            const float v = __fadd_rn(__fadd_rn(u1, u2), al);
-            if (v < inf && dummy_better(v, j1, j2, mine)) mine = DummyBest{v, j1, j2};
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            DummyBest o{__shfl_xor_sync(0xffffffffu, mine.v, off), __shfl_xor_sync(0xffffffffu, mine.j1, off),
-                        __shfl_xor_sync(0xffffffffu, mine.j2, off)};
-            if (dummy_better(o.v, o.j1, o.j2, mine)) mine = o;
-        }
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mine;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            DummyBest best = red[0];
-            for (int w = 1; w < kDummyThreads / 32; ++w)
-                if (dummy_better(red[w].v, red[w].j1, red[w].j2, best)) best = red[w];
-            int32_t *row = assign + un.out_a;
-            if (best.v < inf) {
-                int s2 = best.j1, s1 = best.j2;   // slots of z_{i-2}, z_{i-1}
-                auto out = [&](int i, int s) {
-                    row[md.perm[i]] = s == E ? -2 : sc.perm[cidx[(int64_t)i * K + s]];
-                };
-                out(0, s2);
-                out(1, s1);
-                for (int i = 2; i < M; ++i) {
-                    const int sa = beta[(int64_t)(i - 2) * L * L + s1 * L + s2];
-                    out(i, sa);
-                    s2 = s1;
-                    s1 = sa;
-                }
-                energy[un.out_e] = best.v;
-            } else {
-                for (int i = 0; i < M; ++i) row[i] = -1;
-                energy[un.out_e] = inf;
+
+        // Eq. 13 over (z_1 = c, z_2 = b) in C_1 + eps, C_2 + eps: U + U + alpha_3(z_2, z_1); alpha of the cells with
+        // eps stands where the step i = 2 left it (parity 1)
+        {
+            const List<KM> &L0 = sm.list[0], &L1 = sm.list[1];
+            const int n0 = L0.n, n1 = L1.n;
+            float bv = kInf;
+            int bk = 0x7fffffff;
+            for (int e = tid; e < (KM + 1) * (KM + 1); e += NT) {
+                const int c = e / (KM + 1), b = e % (KM + 1);
+                if (!((c < n0 || c == E) && (b < n1 || b == E))) continue;
+                const float u1 = c == E ? ueps : L0.u[c], u2 = b == E ? ueps : L1.u[b];
+                const float al = c == E ? (b == E ? sm.ee[1] : sm.ea(1, b)) : (b == E ? sm.be(1, c) : sm.alpha[c * AS + b]);
+                argmin_merge(bv, bk, __fadd_rn(__fadd_rn(u1, u2), al), e);
             }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                argmin_merge(bv, bk, __shfl_xor_sync(full, bv, off), __shfl_xor_sync(full, bk, off));
+            if (lane == 0) { sm.red_v[warp] = bv; sm.red_k[warp] = bk; }
+            __syncthreads();
+            if (warp == 0) {
+                bv = sm.red_v[0];
+                bk = sm.red_k[0];
+                for (int w = 1; w < NW; ++w) argmin_merge(bv, bk, sm.red_v[w], sm.red_k[w]);
+                const bool ok = bv < kInf;
+                if (energy && lane == 0) energy[un.out_e] = ok ? bv : kInf;
+                if (assign) {   // Eq. 12, as backtrack_unit: every lane walks, the lanes then write 32 points at once
+                    int32_t *out = assign + un.out_a;
+                    const int z1 = ok ? bk / (KM + 1) : 0, z2 = ok ? bk % (KM + 1) : 0;
+                    int s2 = z1, s1 = z2;
+                    for (int i0 = 0; i0 < M; i0 += 32) {
+                        int mine = kNoSlot;
+                        for (int i = i0; i < min(M, i0 + 32) && ok; ++i) {
+                            int s0 = i == 0 ? z1 : z2;
+                            if (i >= 2) {
+                                s0 = beta[((int64_t)(i - 2) * (KM + 1) + s1) * LS + s2];
+                                s2 = s1;
+                                s1 = s0;
+                            }
+                            if (i - i0 == lane) mine = s0;
+                        }
+                        const int i = i0 + lane;
+                        if (i < M)
+                            out[md.perm[i]] = mine == E ? -2 : mine == kNoSlot ? -1 : sc.perm[cidx[(int64_t)i * K + mine]];
+                    }
+                }
+            }
+            __syncthreads();   // tables, lists and the reduction slots are reused by the next unit
         }
-        __syncthreads();   // tables, lists and the reduction slots are reused by the next unit
     }
     if constexpr (kCount) {
         if (n_eval) atomicAdd(evaluated, n_eval);
     }
 }
 
-}  // namespace
+constexpr int kPerSm64 = 3, kPerSm32 = 4;   // CTAs per SM for lists of up to 64 and 32 candidates
 
-int64_t dummy_scratch_bytes(int K, int max_M, int grid)
+template <int KM, int NT, int MB>
+cudaError_t launch_dummy_t(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes, Params p,
+                           float wd, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
+                           uint8_t *scratch, int64_t per_cta, int grid, int *work_counter, float *energy,
+                           int32_t *assign, unsigned long long *evaluated, cudaStream_t st)
 {
-    const int64_t L = K + 1;
-    return (int64_t)grid * std::max(max_M - 2, 1) * L * L;
+    static_assert(MB * (sizeof(DummySmem<KM, NT>) + 1024) <= 228 * 1024, "shared memory exceeds the CTAs' budget");
+    const size_t smem = sizeof(DummySmem<KM, NT>);
+    auto kern = evaluated ? dummy_recurse_kernel<KM, NT, MB, true> : dummy_recurse_kernel<KM, NT, MB, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(work_counter, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    prof_begin(kProfRecurse, st);
+    kern<<<(unsigned)std::min<int64_t>(n_units, grid), NT, smem, st>>>(units, n_units, models, scenes, p, wd, cand_idx,
+                                                                        cand_u, cand_cnt, scratch, per_cta, work_counter,
+                                                                        energy, assign, evaluated);
+    e = cudaGetLastError();
+    prof_end(kProfRecurse, st);
+    return e;
 }
 
-int dummy_grid()
+int64_t dummy_cta_bytes(int K, int max_M)
+{
+    const int64_t KM = K <= 32 ? 32 : 64;
+    return (std::max(max_M - 2, 1) * (KM + 1) * (KM + 4) + 15) / 16 * 16;
+}
+
+}  // namespace
+
+int64_t dummy_scratch_bytes(int K, int max_M, int grid) { return grid * dummy_cta_bytes(K, max_M); }
+
+int dummy_grid(int K)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                   cudaSuccess)
         return 0;
-    return sms * 2;
+    return sms * (K <= 32 ? kPerSm32 : kPerSm64);
 }
 
 cudaError_t launch_recurse_dummy(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
                                  Params p, float wd, const int32_t *cand_idx, const float *cand_u,
-                                 const int32_t *cand_cnt, uint8_t *scratch, int max_M, int grid, float *energy,
-                                 int32_t *assign, unsigned long long *evaluated, cudaStream_t st)
+                                 const int32_t *cand_cnt, uint8_t *scratch, int max_M, int grid, int *work_counter,
+                                 float *energy, int32_t *assign, unsigned long long *evaluated, cudaStream_t st)
 {
     if (n_units <= 0) return cudaSuccess;
     if (p.K > kMaxK) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(DummySmem);
-    auto kern = evaluated ? dummy_recurse_kernel<true> : dummy_recurse_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int64_t per_cta = (int64_t)std::max(max_M - 2, 1) * (p.K + 1) * (p.K + 1);
-    const int g = (int)std::min<int64_t>(n_units, grid);
-    prof_begin(kProfRecurse, st);
-    kern<<<g, kDummyThreads, smem, st>>>(units, n_units, models, scenes, p, wd, cand_idx, cand_u, cand_cnt, scratch,
-                                         per_cta, energy, assign, evaluated);
-    e = cudaGetLastError();
-    prof_end(kProfRecurse, st);
-    return e;
+    const int64_t per_cta = dummy_cta_bytes(p.K, max_M);
+    if (p.K <= 32)
+        return launch_dummy_t<32, 128, kPerSm32>(units, n_units, models, scenes, p, wd, cand_idx, cand_u, cand_cnt, scratch,
+                                                 per_cta, grid, work_counter, energy, assign, evaluated, st);
+    return launch_dummy_t<64, 256, kPerSm64>(units, n_units, models, scenes, p, wd, cand_idx, cand_u, cand_cnt, scratch,
+                                             per_cta, grid, work_counter, energy, assign, evaluated, st);
 }
 
 }  // namespace hgm
