@@ -738,7 +738,6 @@ hgm_status run_batch(Exec &ex, const hgm_model *const *models, int nm, const hgm
     ex.tensor = pruning || hp->precision == 1;
     if (hp->precision == 1) {
         CK(ws.mnorm.ensure((size_t)R * sizeof(float)), "workspace (norms)");
-        CK(launch_sqnorm_bf16(model_f, R, F, F, ws.mnorm.as<float>(), st), "norm kernel");
     }
 
     // outputs: device pointers are written in place, host ones through staging
@@ -849,7 +848,6 @@ hgm_status run_batch(Exec &ex, const hgm_model *const *models, int nm, const hgm
             const int pts = (int)(sg.j1 - sg.j0);
             float *U = const_cast<float *>(srec[(size_t)g].U);
             if (hp->precision == 1) {
-                CK(launch_sqnorm_bf16(segf, pts, F, F, ws.snorm.as<float>(), st), "norm kernel");
                 CK(launch_unary_bf16(model_f, R, segf, pts, F, F, ws.mnorm.as<float>(),
                                      ws.snorm.as<float>(), p.lambda1, U, srec[(size_t)g].upitch,
                                      ws.status.as<int>(), ws.ubf.p, ws.ubf.bytes, st),
@@ -1037,8 +1035,6 @@ hgm_status single_pair_units(const hgm_model *m, const hgm_scene *s, const hgm_p
         CK(g_ws.snorm.ensure((size_t)std::max(s->d.S, 1) * sizeof(float)), "workspace (norms)");
         CK(g_ws.status.ensure(sizeof(int)), "workspace");
         CK(cudaMemsetAsync(g_ws.status.p, 0, sizeof(int), st), "memset");
-        CK(launch_sqnorm_bf16(m->d.f, R, m->d.F, m->d.F, g_ws.mnorm.as<float>(), st), "norm kernel");
-        CK(launch_sqnorm_bf16(s->d.f, s->d.S, m->d.F, m->d.F, g_ws.snorm.as<float>(), st), "norm kernel");
         CK(g_ws.ubf.ensure(unary_bf16_scratch_bytes(R, s->d.S, m->d.F)), "workspace (BF16 operands)");
         CK(launch_unary_bf16(m->d.f, R, s->d.f, s->d.S, m->d.F, m->d.F, g_ws.mnorm.as<float>(), g_ws.snorm.as<float>(),
                              p.lambda1, g_ws.U.as<float>(), pitch, g_ws.status.as<int>(), g_ws.ubf.p, g_ws.ubf.bytes,
@@ -2158,8 +2154,6 @@ hgm_status hgm_unary_bf16(const hgm_model *model, const hgm_scene *scene, float 
     CK(g_ws.snorm.ensure((size_t)std::max(S, 1) * sizeof(float)), "workspace (norms)");
     CK(g_ws.status.ensure(sizeof(int)), "workspace");
     CK(cudaMemsetAsync(g_ws.status.p, 0, sizeof(int), st), "memset");
-    CK(launch_sqnorm_bf16(model->d.f, M, F, F, g_ws.mnorm.as<float>(), st), "norm kernel");
-    CK(launch_sqnorm_bf16(scene->d.f, S, F, F, g_ws.snorm.as<float>(), st), "norm kernel");
     CK(g_ws.ubf.ensure(unary_bf16_scratch_bytes(M, S, F)), "workspace (BF16 operands)");
     CK(launch_unary_bf16(model->d.f, M, scene->d.f, S, F, F, g_ws.mnorm.as<float>(), g_ws.snorm.as<float>(), lambda1,
                          U, S, g_ws.status.as<int>(), g_ws.ubf.p, g_ws.ubf.bytes, st),

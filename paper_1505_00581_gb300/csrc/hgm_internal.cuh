@@ -131,12 +131,12 @@ cudaError_t launch_collect_infeasible(const UnitResult *res, const Unit *units, 
 cudaError_t launch_unary(const float *A, int R, const float *B, int S, int F, float lambda1, float *U,
                          int ldu, cudaStream_t st);
 // k_rowdot.cu: BF16 tensor-core products.
-cudaError_t launch_sqnorm_bf16(const float *X, int64_t n, int ld, int F, float *out, cudaStream_t st);
+// mnorm [R], snorm [S]: receive the squared norms of the BF16-rounded rows.
 // scratch: device memory of at least unary_bf16_scratch_bytes(R, S, F) for the BF16 copies of the operands
 // the TMA-staged kernel reads (with less, or F > 256, the operands are staged by the threads instead).
 size_t unary_bf16_scratch_bytes(int R, int64_t S, int F);
 cudaError_t launch_unary_bf16(const float *model, int R, const float *scene, int S, int F, int ld,
-                              const float *mnorm, const float *snorm, float lambda1, float *U, int64_t ldu,
+                              float *mnorm, float *snorm, float lambda1, float *U, int64_t ldu,
                               int *status, void *scratch, size_t scratch_bytes, cudaStream_t st);
 cudaError_t launch_rowdot_plain(const float *X, int64_t nrows, int ldx, const float *W, int ncols, int ldw, int F,
                                 const float *bias, float *Y, int64_t ldy, int *status, cudaStream_t st);

@@ -164,21 +164,42 @@ __global__ void __launch_bounds__(128) rowdot_kernel(const float *__restrict__ X
 // stride (LBO) of 2048 bytes and a row-group stride (SBO) of 128 bytes. Every box starts at an inner
 // coordinate that is a multiple of 8 components (16 bytes); rows past the end of a matrix arrive as zeros.
 // A CTA owns 128 scene rows (loaded once) and sweeps the model rows in tiles of 128: one thread issues the
-// B tile's boxes on an mbarrier with the expected byte count, waits, issues the MMAs and commits; the 128
-// threads read the accumulator (thread = scene row) and write U. Two CTAs share an SM, so one's epilogue
-// overlaps the other's copies and MMAs.
+// B tile's boxes on an mbarrier with the expected byte count, waits, issues the MMAs and commits; the 256
+// threads read the accumulator (thread = scene row and half of the columns) and write U. Two CTAs share an SM, so
+// one's epilogue overlaps the other's copies and MMAs. Bound by the latency of a tile's phases, so the model rows are
+// split over the grid until two CTAs per SM have about two turns; 3,264 model x 6,000 scene rows of 162 components:
+// 120 -> 61 us (with 128 threads and runs of eight tiles the grid had 188 CTAs for 304 places).
 
 constexpr uint32_t kTmaLBO = 2048, kTmaSBO = 128;
 
-__global__ void to_bf16_kernel(const float *__restrict__ X, int64_t n, int ld, int F, int Kp,
-                               __nv_bfloat16 *__restrict__ out)
+// Rows of X as BF16 rows of Kp components (zeros after F) and the squared norm of each (FP32, components in order, as
+// bf16_sqnorm_kernel): 32 rows per CTA through shared memory, so that the reads are whole lines and the 32 ordered
+// sums run beside other CTAs' reads. One pass over X instead of two, the second of which had a thread read a row:
+// 6,000 rows of 164 components 21 -> 10 us.
+__global__ void __launch_bounds__(256) rows_to_bf16_kernel(const float *__restrict__ X, int64_t n, int ld, int F, int Kp,
+                                                           __nv_bfloat16 *__restrict__ out, float *__restrict__ norm)
 {
-    const int64_t total = n * (Kp / 2);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / (Kp / 2);
-        const int k = (int)(e - r * (Kp / 2)) * 2;
-        const float a = k < F ? X[r * ld + k] : 0.0f, b = k + 1 < F ? X[r * ld + k + 1] : 0.0f;
-        reinterpret_cast<__nv_bfloat162 *>(out)[e] = __floats2bfloat162_rn(a, b);
+    extern __shared__ float rows[];   // 32 x (Kp + 1) rounded components
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * 32;
+    for (int q = warp; q < 32 && r0 + q < n; q += 8) {
+        const float *x = X + (r0 + q) * ld;
+        __nv_bfloat162 *o = reinterpret_cast<__nv_bfloat162 *>(out + (r0 + q) * Kp);
+        for (int k2 = lane; k2 < Kp / 2; k2 += 32) {
+            const int k = 2 * k2;
+            const __nv_bfloat162 v = __floats2bfloat162_rn(k < F ? x[k] : 0.0f, k + 1 < F ? x[k + 1] : 0.0f);
+            o[k2] = v;
+            rows[q * (Kp + 1) + k] = __bfloat162float(v.x);
+            rows[q * (Kp + 1) + k + 1] = __bfloat162float(v.y);
+        }
+    }
+    __syncthreads();
+    if (warp == 0 && r0 + lane < n) {
+        const float *x = rows + lane * (Kp + 1);
+        float s = 0.0f;
+#pragma unroll 8
+        for (int k = 0; k < F; ++k) s = fmaf(x[k], x[k], s);
+        norm[r0 + lane] = s;
     }
 }
 
@@ -197,7 +218,7 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *tmap, 
         : "memory");
 }
 
-__global__ void __launch_bounds__(128) unary_tma_kernel(const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(256) unary_tma_kernel(const __grid_constant__ CUtensorMap tmA,
                                                         const __grid_constant__ CUtensorMap tmB, int64_t S, int R,
                                                         int Kp, const float *__restrict__ snorm,
                                                         const float *__restrict__ mnorm, float lambda1,
@@ -224,7 +245,9 @@ __global__ void __launch_bounds__(128) unary_tma_kernel(const __grid_constant__ 
     __syncthreads();
     tc05::fence_after_sync();
     const uint32_t taddr = tslot;
-    const uint32_t tlane = taddr + ((uint32_t)(32 * warp) << 16);
+    // a warp reads the TMEM lanes of its quarter of the scene rows, the upper four warps columns 64 to 127
+    const int trow = 32 * (warp & 3) + (tid & 31), col0 = 64 * (warp >> 2);
+    const uint32_t tlane = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
     constexpr uint32_t idesc = tc05::idesc_bf16_f32(TM, TN);
     const int nk8 = Kp / 8;
     const uint32_t tile_bytes = (uint32_t)TM * Kp * 2;
@@ -234,7 +257,7 @@ __global__ void __launch_bounds__(128) unary_tma_kernel(const __grid_constant__ 
     const int m_lo = (int)blockIdx.y * mrows_per_cta, m_hi = min(R, m_lo + mrows_per_cta);
     for (int64_t tile = blockIdx.x; tile < ntiles && !bad; tile += gridDim.x) {
         const int64_t r0 = tile * TM;
-        const int64_t row = r0 + tid;
+        const int64_t row = r0 + trow;
         const float xn = row < S ? snorm[row] : 0.0f;
         for (int m0 = m_lo; m0 < m_hi && !bad; m0 += TN) {
             if (tid == 0) {
@@ -244,7 +267,7 @@ __global__ void __launch_bounds__(128) unary_tma_kernel(const __grid_constant__ 
                     for (int k8 = 0; k8 < nk8; ++k8) tma_load_2d(sA + (size_t)k8 * kTmaLBO, &tmA, 8 * k8, (int)r0, &tma_bar);
                 for (int k8 = 0; k8 < nk8; ++k8) tma_load_2d(sB + (size_t)k8 * kTmaLBO, &tmB, 8 * k8, m0, &tma_bar);
             }
-            wn[tid] = m0 + tid < m_hi ? mnorm[m0 + tid] : 0.0f;
+            if (tid < TN) wn[tid] = m0 + tid < m_hi ? mnorm[m0 + tid] : 0.0f;
             if (tid == 0) {
                 if (tc05::mbar_wait(&tma_bar, tphase, kPolls)) {
                     tc05::fence_after_sync();
@@ -270,7 +293,7 @@ __global__ void __launch_bounds__(128) unary_tma_kernel(const __grid_constant__ 
             mphase ^= 1u;
             tc05::fence_after_sync();
             if (!bad) {
-                for (int cc = 0; cc < TN && m0 + cc < m_hi; cc += 32) {
+                for (int cc = col0; cc < col0 + 64 && m0 + cc < m_hi; cc += 32) {
                     float v[32];
                     tc05::tmem_ld32(tlane + (uint32_t)cc, v);
                     if (row < S) {
@@ -357,7 +380,7 @@ cudaError_t launch_rowdot(const float *X, int64_t nrows, int ldx, const float *W
 
 }  // namespace
 
-cudaError_t launch_sqnorm_bf16(const float *X, int64_t n, int ld, int F, float *out, cudaStream_t st)
+static cudaError_t launch_sqnorm_bf16(const float *X, int64_t n, int ld, int F, float *out, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
     int64_t blocks = std::min<int64_t>((n + 255) / 256, 65535);
@@ -372,7 +395,7 @@ size_t unary_bf16_scratch_bytes(int R, int64_t S, int F)
 }
 
 cudaError_t launch_unary_bf16(const float *model, int R, const float *scene, int S, int F, int ld,
-                              const float *mnorm, const float *snorm, float lambda1, float *U, int64_t ldu,
+                              float *mnorm, float *snorm, float lambda1, float *U, int64_t ldu,
                               int *status, void *scratch, size_t scratch_bytes, cudaStream_t st)
 {
     if (R <= 0 || S <= 0) return cudaSuccess;
@@ -384,31 +407,34 @@ cudaError_t launch_unary_bf16(const float *model, int R, const float *scene, int
     __nv_bfloat16 *sb = mb + (size_t)(R + 255) / 256 * 256 * Kp;
     if (Kp <= KC && scratch && scratch_bytes >= unary_bf16_scratch_bytes(R, S, F) &&
         encode_rows(&tmA, sb, S, Kp) && encode_rows(&tmB, mb, R, Kp)) {
-        // BF16 copies of both operands, then the TMA-staged contraction
-        const int64_t bm = std::min<int64_t>(((int64_t)R * Kp / 2 + 255) / 256, 65536);
-        const int64_t bs = std::min<int64_t>(((int64_t)S * Kp / 2 + 255) / 256, 65536);
-        to_bf16_kernel<<<(unsigned)bm, 256, 0, st>>>(model, R, ld, F, Kp, mb);
-        to_bf16_kernel<<<(unsigned)bs, 256, 0, st>>>(scene, S, ld, F, Kp, sb);
+        // BF16 copies of both operands and their norms, then the TMA-staged contraction
+        const size_t rows_smem = (size_t)32 * (Kp + 1) * sizeof(float);
+        rows_to_bf16_kernel<<<(unsigned)((R + 31) / 32), 256, rows_smem, st>>>(model, R, ld, F, Kp, mb, mnorm);
+        rows_to_bf16_kernel<<<(unsigned)(((int64_t)S + 31) / 32), 256, rows_smem, st>>>(scene, S, ld, F, Kp, sb, snorm);
         const size_t smem = (size_t)2 * TM * Kp * 2 + 1024;
         e = cudaFuncSetAttribute(unary_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int dev = 0, sms = 0, per_sm = 0;
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, unary_tma_kernel, 128, smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, unary_tma_kernel, 256, smem);
         if (e == cudaSuccess) {
             per_sm = per_sm < 1 ? 1 : (per_sm > 4 ? 4 : per_sm);   // 4 x 128 TMEM columns = the SM's 512
-            // scene tiles on x, chunks of kMTiles model tiles on y: enough CTAs that two per SM overlap one
-            // another's copies, products and epilogues even when the scene has few tiles
-            constexpr int kMTiles = 8;
-            const int64_t stiles = ((int64_t)S + TM - 1) / TM;
-            const int mchunks = (R + TN * kMTiles - 1) / (TN * kMTiles);
+            // scene tiles on x, runs of model tiles on y: as few runs as give two turns of the chip's CTAs, since every
+            // run stages its scene tile again
+            const int64_t stiles = ((int64_t)S + TM - 1) / TM, mtiles = ((int64_t)R + TN - 1) / TN;
+            const int64_t turns = (int64_t)sms * per_sm * 2;
+            const int64_t run = std::max<int64_t>(1, std::min<int64_t>(mtiles, stiles * mtiles / turns));
+            const int64_t mchunks = std::min<int64_t>((mtiles + run - 1) / run, 65535);
+            const int64_t rows_per = (mtiles + mchunks - 1) / mchunks * TN;
             const int64_t gx = std::min<int64_t>(stiles, std::max<int64_t>(1, (int64_t)sms * per_sm * 8 / mchunks));
-            unary_tma_kernel<<<dim3((unsigned)gx, (unsigned)mchunks), 128, smem, st>>>(
-                tmA, tmB, S, R, Kp, snorm, mnorm, lambda1, U, ldu, TN * kMTiles, status);
+            unary_tma_kernel<<<dim3((unsigned)gx, (unsigned)mchunks), 256, smem, st>>>(
+                tmA, tmB, S, R, Kp, snorm, mnorm, lambda1, U, ldu, (int)rows_per, status);
             e = cudaGetLastError();
         }
     } else {
-        e = launch_rowdot<kDist>(scene, S, ld, model, R, ld, F, snorm, mnorm, lambda1, nullptr, U, ldu, status, st);
+        e = launch_sqnorm_bf16(model, R, ld, F, mnorm, st);
+        if (e == cudaSuccess) e = launch_sqnorm_bf16(scene, S, ld, F, snorm, st);
+        if (e == cudaSuccess) e = launch_rowdot<kDist>(scene, S, ld, model, R, ld, F, snorm, mnorm, lambda1, nullptr, U, ldu, status, st);
     }
     prof_end(kProfUnary, st);
     return e;
