@@ -64,3 +64,26 @@ def test_few_and_many_units_give_the_same_bits(env, K):
         f1, e1, a1 = hgm.match(m, s, p)
         assert f1 == lo and len(e1) == n
         assert np.array_equal(e1, e[lo - first:lo - first + n]) and np.array_equal(a1, a[lo - first:lo - first + n])
+
+
+@pytest.mark.parametrize("K,lam,crowd,T,window,M", [
+    (1, 3.0, 0.0, 10, 1, 5), (5, 6.0, 0.2, 10, 2, 9), (8, 20.0, 0.0, 4, 2, 8), (9, 8.0, 0.1, 10, 2, 10),
+    (13, 20.0, 0.3, 0, 2, 7), (16, 30.0, 0.0, 10, 1, 3), (16, 1.0, 0.2, 10, 3, 20), (15, 12.0, 0.0, 2, 3, 9)])
+def test_short_list_edges(env, K, lam, crowd, T, window, M):
+    """The short-list kernel (caps up to 8 and up to 16) as above; the caps the large kernel takes next give the same
+    optimum where no list is cut by either (tested through the oracle)."""
+    test_list_edges(env, K, lam, crowd, T, window, M)
+
+
+@pytest.mark.parametrize("K", [8, 16])
+def test_short_lists_few_and_many_units(env, K):
+    test_few_and_many_units_give_the_same_bits(env, K)
+    torch, hgm, oracle = env
+    rng = np.random.default_rng(K)
+    mod = synth.make_model(rng, 12, F=16, frame=(60.0, 40.0), t_span=10)
+    sc = _scene(rng, mod, 2500, 6.0, 0.0)       # more units than the four-warp form takes
+    m, s = hgm.Model(mod.xy, mod.t, mod.f), hgm.Scene(sc.xy, sc.t, sc.f, sc.n_frames)
+    first, e, a = hgm.match(m, s, hgm.default_params(K=K, window=3))
+    p = hgm.default_params(K=K, window=3, offset_lo=first + 1000, offset_hi=first + 1099)
+    f1, e1, a1 = hgm.match(m, s, p)
+    assert np.array_equal(e1, e[1000:1100]) and np.array_equal(a1, a[1000:1100])
