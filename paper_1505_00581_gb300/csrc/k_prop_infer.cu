@@ -41,13 +41,21 @@ constexpr float kNegInf = -__builtin_huge_valf();
 
 constexpr uint32_t kSBO16 = 2 * 128;       // K = 16 components per row (the bias block)
 
+// The A tiles: core matrices (8 rows x 16 bytes) of one K chunk follow one another down the rows, and chunks
+// are 16 bytes further apart than their 16 core matrices take. A warp writes 4 rows x 8 neighbouring chunks at
+// a time, eight lanes to a row, so the eight lanes of a row fall on all 32 banks once.
+constexpr uint32_t kALBO = (TM / 8) * 128 + 16;
+constexpr uint32_t kASBO = 128;
+constexpr uint32_t kATile = (H / 8) * kALBO;
+
 struct Smem {
-    unsigned char a[2][TM * H * 2];  // hidden layer 1 of two tiles, BF16, canonical K-major
+    unsigned char a[2][kATile];      // hidden layer 1 of two tiles, BF16, K-major, strides kALBO and kASBO
     unsigned char w2[H * H * 2];     // W2 (rows = output units), BF16
     // the layer-2 bias as a 17th K step of the MMA: A gets a constant block (component 0 = 1, the rest 0)
     // shared by both tiles, W2 a block whose component 0 is b2 (BF16)
     unsigned char a1[TM * 16 * 2];
     unsigned char b2k[H * 16 * 2];
+    int2 meta[2][TM];                // per row of a tile: Q row of its candidate (-1 none), its dt as a BF16 pair
     float part[2][2][TM];            // [buffer][column half][row]: half-sums of the last layer
     float w3[H];                     // output weights
     float b3;
@@ -74,10 +82,14 @@ __global__ void fold_xy_kernel(float *__restrict__ rows, int64_t n, const float2
 }
 
 // Final logit of every candidate of every list: scores [n_lists x K] (-inf for empty slots).
-// 256 threads. Building a tile: warp w owns hidden units [32 (w%4), +32) of rows [64 (w/4), +64); lane l
-// takes row 8g + l/4 of each group g of 8 and the 8 units 32 (w%4) + 8 (l%4) .. +8, so a warp reads 8 BF16
-// Q rows as whole 32-byte sectors and writes 4 contiguous core matrices of the A tile. Epilogue: row
+// 256 threads. Building a tile: warp w owns hidden units [64 (w%2), +64) of rows [32 (w/2), +32); lane l takes
+// row 4g + l/8 of each group g of 4 and the 8 units 64 (w%2) + 8 (l%8) .. +8, so a warp reads 4 BF16 Q rows by
+// whole 128-byte lines. What a row needs besides (its candidate's Q row and dt) is looked up once, by thread
+// tid = row, one tile ahead, its index two tiles ahead, and passed on through shared memory. Epilogue: row
 // r = tid % 128, half = tid / 128 owns accumulator columns [64 half, 64 half + 64).
+// The shared-memory/L1 pipe bounds the kernel. Reading half lines (8 rows x 64 bytes), looking indices, counts
+// and frames up once per row and warp, and storing the tile with four lanes of a row on the same banks:
+// 522,000 lists of 64 (34 M candidates, 8.5 GB of Q lines through L2) take 2.20 ms, 3.9 TB/s; 2.93 ms before.
 __global__ void __launch_bounds__(256, 2) prop_score_kernel(const Unit *__restrict__ units, int64_t n_units,
                                                             const ModelRec *__restrict__ models,
                                                             const SceneRec *__restrict__ scenes, Params p,
@@ -94,10 +106,8 @@ __global__ void __launch_bounds__(256, 2) prop_score_kernel(const Unit *__restri
     const int lpt = TM >> kp_log2;                                  // lists per tile
     const int lsub = row >> kp_log2, slot = row & ((1 << kp_log2) - 1);
     // build-phase roles
-    // a row's four 16-byte chunks sit on adjacent lanes (measured faster for the gathers than the
-    // bank-conflict-free order of the A-tile stores)
-    const int bh0 = 32 * (warp & 3) + 8 * (lane & 3);              // first of this lane's 8 hidden units
-    const int brow0 = 64 * (warp >> 2) + (lane >> 2);                // its row in group 0 (+8 per group)
+    const int bh0 = 64 * (warp & 1) + 8 * (lane & 7);              // first of this lane's 8 hidden units
+    const int brow0 = 32 * (warp >> 1) + (lane >> 3);                // its row in group 0 (+4 per group)
     __nv_bfloat162 w1t[4];                                           // W1c_t / w for those units, BF16 pairs
 #pragma unroll
     for (int e = 0; e < 4; ++e)
@@ -181,62 +191,67 @@ __global__ void __launch_bounds__(256, 2) prop_score_kernel(const Unit *__restri
         if (o >= 0) scores[o] = v ? sm.b3 + sm.part[b][0][row] + sm.part[b][1][row] : kNegInf;
     };
 
-    for (int64_t u = blockIdx.x; u < n_units && !stop; u += gridDim.x) {
+    // units come longest first: rounds run over the CTAs back and forth, which evens out their sums
+    for (int64_t u0 = 0, odd = 0; u0 < n_units && !stop; u0 += gridDim.x, odd ^= 1) {
+        const int64_t u = u0 + (odd ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+        if (u >= n_units) continue;
         const Unit un = units[u];
         const ModelRec md = models[un.model];
         const SceneRec sc = scenes[un.scene];
         const int M = md.M;
         const int64_t lbase = un.cand / K;
-        // the 8 row groups' list counts and raw candidate indices of the tile at i0 (the slot clamped into the
-        // unit's lists, so the index load does not wait for the count); the next tile's are loaded right after
-        // this tile's build, so that they arrive while the barrier, the MMA issue and the epilogue run
-        int cn[8], jr[8];
-        auto load_idx = [&](int i0n) {
-#pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                const int r = brow0 + 8 * g, lst = i0n + (r >> kp_log2), sl = r & ((1 << kp_log2) - 1);
-                const int lc = lst < M ? lst : M - 1, sc_ = sl < K ? sl : K - 1;
-                cn[g] = cand_cnt[lbase + lc];
-                jr[g] = cand_idx[un.cand + (int64_t)lc * K + sc_];
-            }
+        // half 0: candidate of this thread's row in the tile at i0n (-1 none; the slot is clamped into the unit's
+        // lists, so the index load does not wait for the count), and the row's entry of a tile's table
+        auto candidate = [&](int i0n) {
+            const int lst = i0n + lsub, lc = lst < M ? lst : M - 1;
+            const int c = cand_cnt[lbase + lc];
+            const int j = cand_idx[un.cand + (int64_t)lc * K + (slot < K ? slot : K - 1)];
+            return lst < M && slot < c ? j : -1;
         };
-        load_idx(0);
+        auto row_dt = [&](int j, int i0n) { return j >= 0 ? sc.t[j] - md.t[i0n + lsub] - un.offset : 0; };
+        auto put_meta = [&](int b, int j, int dt) {
+            const __nv_bfloat162 d2 = __float2bfloat162_rn((float)dt);
+            sm.meta[b][row] = make_int2(j >= 0 ? j - sc.ucol0 : -1, (int)*reinterpret_cast<const uint32_t *>(&d2));
+        };
+        int jc = -1, jn = -1;   // the row's candidate in this tile and in the next
+        if (half == 0) {
+            jc = candidate(0);
+            if (lpt < M) jn = candidate(lpt);
+            put_meta((int)(k & 1), jc, row_dt(jc, 0));   // last read before the barrier of tile k-2
+        }
+        __syncthreads();
         for (int i0 = 0; i0 < M; i0 += lpt) {
             const int buf = (int)(k & 1);
             unsigned char *arow = sm.a[buf];
-            // gather: the candidate indices (loaded before), then their frames and Q chunks
-            int jg[8];
-            bool vg[8];
-#pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                const int r = brow0 + 8 * g, lst = i0 + (r >> kp_log2), sl = r & ((1 << kp_log2) - 1);
-                vg[g] = lst < M && sl < cn[g];
-                jg[g] = vg[g] ? jr[g] : 0;
+            int dtn = 0, jnn = -1;
+            if (half == 0 && i0 + lpt < M) {
+                dtn = row_dt(jn, i0 + lpt);
+                if (i0 + 2 * lpt < M) jnn = candidate(i0 + 2 * lpt);
             }
-            int tg[8];
+            int2 mg[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) mg[g] = sm.meta[buf][brow0 + 4 * g];
+            // (asking for the next tile's chunks here, before the epilogue of the last, changed nothing: 8.88 and
+            // 8.86 ms of a pruned batch)
             uint4 qg[8];
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
-                if (vg[g]) {
-                    tg[g] = sc.t[jg[g]];
-                    qg[g] = __ldg(reinterpret_cast<const uint4 *>(sc.pq + (int64_t)(jg[g] - sc.ucol0) * H + bh0));
-                } else {
-                    tg[g] = 0;
-                    qg[g] = make_uint4(0, 0, 0, 0);
-                }
+                qg[g] = make_uint4(0, 0, 0, 0);
+                if (mg[g].x >= 0)
+                    qg[g] = __ldg(reinterpret_cast<const uint4 *>(sc.pq + (int64_t)mg[g].x * H + bh0));
             }
             int plist = -1;
             uint4 pv = make_uint4(0, 0, 0, 0);
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
-                const int r = brow0 + 8 * g, lst = i0 + (r >> kp_log2);
+                const int r = brow0 + 4 * g, lst = i0 + (r >> kp_log2);
                 __align__(16) __nv_bfloat162 hh[4];
-                if (vg[g]) {
+                if (mg[g].x >= 0) {
                     if (lst != plist) {   // the row's list: this lane's 8 units of P (rows of a group share it)
                         pv = __ldg(reinterpret_cast<const uint4 *>(pi.Pb + (int64_t)(md.urow + lst) * H + bh0));
                         plist = lst;
                     }
-                    const __nv_bfloat162 dt = __float2bfloat162_rn((float)(tg[g] - md.t[lst] - un.offset));
+                    const __nv_bfloat162 dt = *reinterpret_cast<const __nv_bfloat162 *>(&mg[g].y);
                     const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(&pv);
                     const __nv_bfloat162 *q2 = reinterpret_cast<const __nv_bfloat162 *>(&qg[g]);
 #pragma unroll
@@ -246,13 +261,15 @@ __global__ void __launch_bounds__(256, 2) prop_score_kernel(const Unit *__restri
 #pragma unroll
                     for (int e = 0; e < 4; ++e) hh[e] = __floats2bfloat162_rn(0.0f, 0.0f);
                 }
-                *reinterpret_cast<uint4 *>(arow + tc05::kmajor_offset(r, bh0, kLBO, kSBO)) =
+                *reinterpret_cast<uint4 *>(arow + tc05::kmajor_offset(r, bh0, kALBO, kASBO)) =
                     *reinterpret_cast<uint4 *>(hh);
             }
-            if (i0 + lpt < M) load_idx(i0 + lpt);
+            if (half == 0 && i0 + lpt < M) put_meta(buf ^ 1, jn, dtn);   // last read before the barrier of tile k-1
             // this thread's epilogue row
             const int list = i0 + lsub;
-            const bool valid = list < M && slot < cand_cnt[lbase + (list < M ? list : 0)];
+            const bool valid = jc >= 0;
+            jc = jn;
+            jn = jnn;
             const int64_t o0 = (half == 0 && list < M && slot < K) ? (lbase + list) * K + slot : -1;
             tc05::fence_proxy_async_smem();
             tc05::fence_before_sync();
@@ -263,7 +280,7 @@ __global__ void __launch_bounds__(256, 2) prop_score_kernel(const Unit *__restri
             if (tid == 0) {
                 const uint32_t a0 = tc05::smem_u32(arow), b0 = tc05::smem_u32(sm.w2);
                 for (int ks = 0; ks < H / 16; ++ks)
-                    tc05::mma_bf16(taddr + (uint32_t)(H * buf), tc05::smem_desc(a0 + ks * 2 * kLBO, kLBO, kSBO),
+                    tc05::mma_bf16(taddr + (uint32_t)(H * buf), tc05::smem_desc(a0 + ks * 2 * kALBO, kALBO, kASBO),
                                    tc05::smem_desc(b0 + ks * 2 * kLBO, kLBO, kSBO), idesc, ks > 0);
                 tc05::mma_bf16(taddr + (uint32_t)(H * buf), tc05::smem_desc(tc05::smem_u32(sm.a1), kLBO, kSBO16),
                                tc05::smem_desc(tc05::smem_u32(sm.b2k), kLBO, kSBO16), idesc, true);
@@ -298,7 +315,9 @@ __global__ void __launch_bounds__(256, 2) prop_score_kernel(const Unit *__restri
 }
 
 // Per (unit, i) list: keep the `keep` best scores (ties: lower slot), in slot order, with their FP32 unary
-// costs from the candidate list (re-scored afterwards in the precision mode). One warp per list.
+// costs from the candidate list (re-scored afterwards in the precision mode). One warp per list. Bound by
+// instruction issue: keep 16 of 522,000 lists of 64 took 413 us when every differing bit of the keys was tried,
+// 249 us stopping at a threshold that separates the kept from the rest.
 __global__ void __launch_bounds__(256) prop_keep_kernel(const Unit *__restrict__ units, int64_t n_units,
                                                         const ModelRec *__restrict__ models, Params p, int keep,
                                                         const float *__restrict__ scores,
@@ -320,25 +339,8 @@ __global__ void __launch_bounds__(256) prop_keep_kernel(const Unit *__restrict__
             const int nl = cand_cnt[lbase + li];
             const int kk = nl < keep ? nl : keep;
             const float *sl = scores + (lbase + li) * K;
-            bool c0 = false, c1 = false;
-            if (kk <= 10) {
-                // a few rounds of a warp-wide argmax (ties: lower slot); longer keeps bisect for the threshold
-                float v0 = lane < nl ? sl[lane] : kNegInf;
-                float v1 = lane + 32 < nl ? sl[lane + 32] : kNegInf;
-                for (int q = 0; q < kk; ++q) {
-                    float bv = v0 >= v1 ? v0 : v1;
-                    int bs = v0 >= v1 ? lane : lane + 32;
-                    if (lane >= nl) bs = 1 << 20;
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-                        const int os = __shfl_xor_sync(0xffffffffu, bs, off);
-                        if (ov > bv || (ov == bv && os < bs)) { bv = ov; bs = os; }
-                    }
-                    if (bs == lane) { c0 = true; v0 = kNegInf; }
-                    if (bs == lane + 32) { c1 = true; v1 = kNegInf; }
-                }
-            } else {
+            bool c0 = lane < nl, c1 = lane + 32 < nl;
+            if (kk < nl) {
                 // the kept set: the kk largest scores, ties to the lower slot (slots in [0, nl)). Scores become
                 // order-preserving keys (larger score, larger key); empty slots get key 0, below every score's key
                 // (a score is finite or -inf, whose key is 0x007fffff)
@@ -348,23 +350,23 @@ __global__ void __launch_bounds__(256) prop_keep_kernel(const Unit *__restrict__
                 };
                 const uint32_t k0 = lane < nl ? okey(sl[lane]) : 0u;
                 const uint32_t k1 = lane + 32 < nl ? okey(sl[lane + 32]) : 0u;
-                // the kk-th largest key T, bit by bit from the top: the largest T with at least kk keys >= T.
-                // Bits on which every key of the list agrees are read off an AND and an OR of the keys.
-                uint32_t kand = k0 & k1, kor = k0 | k1;
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    kand &= __shfl_xor_sync(0xffffffffu, kand, off);
-                    kor |= __shfl_xor_sync(0xffffffffu, kor, off);
-                }
+                // the largest T with at least kk keys >= T, bit by bit from the top. Bits on which every key of the
+                // list agrees are read off an AND and an OR of the keys; the search ends as soon as exactly kk keys
+                // are >= T, which takes about log2 of the list's length in steps after the first differing bit, where
+                // the kk-th key itself would take every differing bit (more than twenty)
+                const uint32_t kand = __reduce_and_sync(0xffffffffu, (lane < nl ? k0 : 0xffffffffu) &
+                                                                         (lane + 32 < nl ? k1 : 0xffffffffu));
+                const uint32_t kor = __reduce_or_sync(0xffffffffu, k0 | k1);
                 const uint32_t differ = kand ^ kor;
-                uint32_t T = kand & ~differ;   // the common bits
-                // only the differing bits need a test, from the highest down
-                for (int bit = differ ? 31 - __clz(differ) : -1; bit >= 0; --bit) {
-                    if (!((differ >> bit) & 1u)) continue;
-                    const uint32_t cand = T | (1u << bit);
+                uint32_t T = kand;             // the common bits
+                for (uint32_t rest = differ; rest;) {
+                    const uint32_t bit = 0x80000000u >> __clz(rest);
+                    rest ^= bit;
+                    const uint32_t cand = T | bit;
                     const int cnt = __popc(__ballot_sync(0xffffffffu, k0 >= cand)) +
                                     __popc(__ballot_sync(0xffffffffu, k1 >= cand));
                     if (cnt >= kk) T = cand;
+                    if (cnt == kk) break;
                 }
                 // keep every key above T, then the keys equal to T in slot order up to kk
                 const int above =
@@ -522,7 +524,7 @@ cudaError_t launch_prop_score(const Unit *units, int64_t n_units, const ModelRec
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    // two CTAs per SM: 2 x ~101 KB of shared memory, 2 x 256 of the SM's 512 TMEM columns
+    // two CTAs per SM: 2 x ~110 KB of shared memory, 2 x 256 of the SM's 512 TMEM columns
     const int64_t grid = std::min<int64_t>(n_units, (int64_t)sms * 2);
     prop_score_kernel<<<(unsigned)grid, 256, smem, st>>>(units, n_units, models, scenes, p, pi, kp_log2, cand_idx,
                                                          cand_cnt, scores, status);
