@@ -51,13 +51,15 @@
 #include <algorithm>
 #include <climits>
 
+#include <cooperative_groups.h>
+
 #include "backtrack.cuh"
 #include "recurse_lists.cuh"
 
 namespace hgm {
 namespace {
 
-template <int KM, int NT>
+template <int KM, int NT, int CL>
 struct Smem {
     // row strides: rows of different b read at the same place fall into different banks (FS, SS); rows of r and
     // alpha are whole 16-byte groups whose starts are 4 banks apart, and their four words past the KM columns hold
@@ -65,12 +67,14 @@ struct Smem {
     static constexpr int FS = KM + 1, SS = KM + 4, RS = KM + 4, AS = KM + 4;
     float2 fb[KM * FS];                   // per b: kept (base, p1) in increasing a
     float r[KM * RS];                     // theta(a->c) or +inf, at a*RS + c | 16 bytes of tile_b per row
-    float alpha[KM * AS];                 // base(a,b) of the coming step at b*AS + a | rank key, tile info of b
+    // base(a,b) of the coming step at b*AS + a | rank key, tile info of b; a cluster's CTAs write one another's rows
+    // of the next step while this one's are still read (step i: half i & 1)
+    float alpha[(CL > 1 ? 2 : 1) * KM * AS];
     uint8_t fs[KM * SS];                  // slot a of each kept entry, | 0x80 when a lies at b's position
     List<KM> list[3];
     float4 geo[2];                        // model constants of step i at geo[i & 1]
-    float red_v[NT / 32];
-    int32_t red_k[NT / 32];
+    float red_v[CL * NT / 32];
+    int32_t red_k[CL * NT / 32];
     int32_t ntile;                        // tiles of the step
     int32_t unit;
     int32_t coin[2];                      // step i: some kept a lies at its b's position (coin[i & 1])
@@ -82,6 +86,37 @@ struct Smem {
     __device__ int32_t &info(int b) { return reinterpret_cast<int32_t *>(alpha)[b * AS + KM + 1]; }
 };
 
+// A warp's searches of a list's first n (<= KM) entries: how many of an ascending array lie below x, and the slot
+// that holds x (KM: none).
+template <int KM>
+__device__ __forceinline__ int entries_below(const int32_t *arr, int n, int x, int lane)
+{
+    int c = 0;
+#pragma unroll
+    for (int k = 0; k < KM; k += 32) c += __popc(__ballot_sync(0xffffffffu, k + lane < n && arr[k + lane] < x));
+    return c;
+}
+
+template <int KM>
+__device__ __forceinline__ int entry_at(const int32_t *arr, int n, int x, int lane)
+{
+    int f = KM;
+#pragma unroll
+    for (int k = KM - 32; k >= 0; k -= 32) {
+        const unsigned m = __ballot_sync(0xffffffffu, k + lane < n && arr[k + lane] == x);
+        if (m) f = k + __ffs((int)m) - 1;
+    }
+    return f;
+}
+
+// The smallest of a warp's values (order-preserving keys; a NaN counts as +inf, as fminf takes it).
+__device__ __forceinline__ float warp_min(float x)
+{
+    const uint32_t u = __float_as_uint(fminf(x, kInf));
+    const uint32_t k = __reduce_min_sync(0xffffffffu, (u >> 31) ? ~u : (u | 0x80000000u));
+    return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k);
+}
+
 // kCount = true builds the accounting variant: identical work, plus a count of
 // the (a, b, c) evaluations the triple loop performs (kept a x CT per tile).
 // kFused = true builds the self-contained variant used for the exact fallback
@@ -90,7 +125,10 @@ struct Smem {
 // live in a per-CTA scratch block (beta + blockIdx.x * beta_cta, reused unit
 // after unit), and the CTA backtracks its own unit and writes the energy and
 // the assignment itself.
-template <int KM, int NT, int MB, int CT, int UR, bool kCount, bool kFused>
+// CL > 1 builds the variant in which a cluster of CL CTAs shares a unit: CTA r owns the rows b with b % CL == r, their
+// kept lists and their tiles, holds the theta(a->c) table whole, and writes a cell's base into the next step's row c
+// in the shared memory of that row's owner; one cluster barrier per step takes the place of the last CTA barrier.
+template <int KM, int NT, int MB, int CT, int UR, bool kCount, bool kFused, int CL>
 __global__ void __launch_bounds__(NT, MB)
 recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *__restrict__ models,
                const SceneRec *__restrict__ scenes, Params p, const int32_t *__restrict__ cand_idx,
@@ -106,13 +144,16 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
     }
     unsigned long long n_eval = 0;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using SM = Smem<KM, NT>;
+    using SM = Smem<KM, NT, CL>;
     SM &sm = *reinterpret_cast<SM *>(smem_raw);
     constexpr int RS = SM::RS, AS = SM::AS, FS = SM::FS, SS = SM::SS;
     constexpr int NW = NT / 32;
-    constexpr int TPB = NT / KM;           // threads per b (and per c): neighbouring lanes
+    constexpr int TPC = NT / KM;           // threads per c: neighbouring lanes
+    constexpr int TPB = TPC * CL;          // threads per b of the CTA's rows
     constexpr int AH = KM / TPB;           // slots a per thread: a = AH h + 0 .. AH - 1
-    static_assert(TPB == 4 || TPB == 8, "threads per b");
+    static_assert(CL == 1 ? TPB == 4 || TPB == 8 : TPB == 32, "threads per b");
+    constexpr bool kWarpRow = TPB == 32;   // a warp per b: ballots in place of searches and exchanges
+    constexpr int kHalf = CL > 1 ? KM * AS : 0;
     const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = p.K;
@@ -120,14 +161,28 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
     const float lam2 = p.lambda2;
     const float lam23 = p.lambda2 * p.lambda3;
     const float gmax = lam23 * kGeoMax;
-    const int h = tid % TPB, row = tid / TPB;
+    unsigned rank = 0;
+    int64_t u_next = 0;                    // CL > 1: units go to the clusters in turn
+    if constexpr (CL > 1) {
+        rank = cooperative_groups::this_cluster().block_rank();
+        u_next = blockIdx.x / CL;
+        cooperative_groups::this_cluster().sync();   // every CTA runs before its memory is written
+    }
+    const int h = tid % TPB, row = tid / TPB * CL + (int)rank;
+    const int hc = tid % TPC, rowc = tid / TPC;
     // a thread reads its run of slots from a start of its own, so that a warp's reads hit every bank once
-    const int rot = TPB == 4 ? h : (h & 1) + ((h >> 2) << 1);
+    const int rot = TPB == 4 ? h : TPB == 8 ? (h & 1) + ((h >> 2) << 1) : 0;
 
     for (;;) {
-        if (tid == 0) sm.unit = atomicAdd(work_counter, 1);
-        __syncthreads();
-        const int64_t u = sm.unit;
+        int64_t u;
+        if constexpr (CL > 1) {
+            u = u_next;
+            u_next += gridDim.x / CL;
+        } else {
+            if (tid == 0) sm.unit = atomicAdd(work_counter, 1);
+            __syncthreads();
+            u = sm.unit;
+        }
         if (u >= n_units) {
             if constexpr (kCount) atomicAdd(evaluated, n_eval);
             break;
@@ -139,7 +194,7 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
         const int32_t *cidx = cand_idx + un.cand;
         const float *cu = cand_u + un.cand;
         const int32_t *ccnt = cand_cnt + un.cand / K;
-        uint8_t *ubeta = kFused ? beta + (int64_t)blockIdx.x * beta_cta : beta + un.beta;
+        uint8_t *ubeta = kFused ? beta + (int64_t)(blockIdx.x / CL) * beta_cta : beta + un.beta;
 
         // the three lists and the constants of the first step
         for (int q = 1; q <= 3 && q <= M; ++q)
@@ -153,12 +208,15 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
         {   // the first step's base: alpha_{M+1} == 0 (Eq. 11)
             const List<KM> &LA = sm.list[(M - 1) % 3], &LB = sm.list[(M - 2) % 3];
             const int dt_ab = __float_as_int(sm.geo[(M - 1) & 1].z);
-            for (int e = tid; e < KM * KM; e += NT) {
-                const int b = e / KM, a = e % KM;
+            float *first = sm.alpha + ((M - 1) & 1) * kHalf;
+            for (int e = tid; e < KM * KM / CL; e += NT) {
+                const int b = e / KM * CL + (int)rank, a = e % KM;
                 // slots past a list hold t = 0x3fffffff, idx = -1, u = inf
                 const bool ok = a < LA.n && b < LB.n && LA.t[a] >= LB.t[b] && LA.idx[a] != LB.idx[b];
-                sm.alpha[b * AS + a] = ok ? base_cost(LA.u[a], lam2, dt_ab, LA.t[a], LB.t[b], 0.0f) : kInf;
+                first[b * AS + a] = ok ? base_cost(LA.u[a], lam2, dt_ab, LA.t[a], LB.t[b], 0.0f) : kInf;
             }
+            if constexpr (CL > 1)   // the other CTAs' rows have no tiles here
+                for (int b = tid; b < KM; b += NT) sm.key(b) = 0;
         }
         __syncthreads();
 
@@ -194,14 +252,18 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                 float2 pb = make_float2(0.f, 0.f);
                 int tb = 0, ib = -1;
                 if (inb) { pb = LB.xy[b]; tb = LB.t[b]; ib = LB.idx[b]; }
-                const float *arow = sm.alpha + b * AS + AH * h;
+                const float *arow = sm.alpha + (i & 1) * kHalf + b * AS + AH * h;
                 // the a with t'(a) >= t'(b) form a suffix of list A (time order): the slots before it are never
                 // feasible with b, and the row holds nothing of this step there
                 int lo = 0;
-                for (int hi = inb ? na : 0; lo < hi;) {
-                    const int mid = (lo + hi) >> 1;
-                    if (LA.t[mid] < tb) lo = mid + 1;
-                    else hi = mid;
+                if constexpr (kWarpRow) {
+                    if (inb) lo = entries_below<KM>(LA.t, na, tb, lane);
+                } else {
+                    for (int hi = inb ? na : 0; lo < hi;) {
+                        const int mid = (lo + hi) >> 1;
+                        if (LA.t[mid] < tb) lo = mid + 1;
+                        else hi = mid;
+                    }
                 }
                 const int j0 = lo - AH * h, j1 = (inb ? na : 0) - AH * h;
                 // smallest and second smallest base over all feasible a
@@ -214,15 +276,22 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     m2 = fminf(m2, fmaxf(m1, v[k]));
                     m1 = fminf(m1, v[k]);
                 }
-#pragma unroll
-                for (int off = 1; off < TPB; off <<= 1) {
-                    const float o1 = __shfl_xor_sync(full, m1, off), o2 = __shfl_xor_sync(full, m2, off);
-                    m2 = fminf(fmaxf(m1, o1), fminf(m2, o2));
-                    m1 = fminf(m1, o1);
-                }
                 // lowest slot of a value among the row's (1 << 20: none)
                 auto slot_of_value = [&](float x, int skip) {
                     int s = 1 << 20;
+                    if constexpr (kWarpRow) {
+                        unsigned has = 0, at[AH];
+#pragma unroll
+                        for (int k = 0; k < AH; ++k) {
+                            at[k] = __ballot_sync(full, v[k] == x && AH * h + k != skip);
+                            has |= at[k];
+                        }
+                        const int f = __ffs((int)has) - 1;
+#pragma unroll
+                        for (int k = AH - 1; k >= 0; --k)
+                            if (has && (at[k] >> f) & 1u) s = AH * f + k;
+                        return s;
+                    }
 #pragma unroll
                     for (int k = 0; k < AH; ++k) {
                         const int a = AH * h + ((k + rot) & (AH - 1));
@@ -232,8 +301,22 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     for (int off = 1; off < TPB; off <<= 1) s = min(s, __shfl_xor_sync(full, s, off));
                     return s;
                 };
+                int s1;
+                if constexpr (kWarpRow) {
+                    const float own1 = m1, own2 = m2;
+                    m1 = warp_min(own1);
+                    s1 = slot_of_value(m1, -1);
+                    m2 = warp_min(s1 / AH == h ? own2 : own1);
+                } else {
+#pragma unroll
+                    for (int off = 1; off < TPB; off <<= 1) {
+                        const float o1 = __shfl_xor_sync(full, m1, off), o2 = __shfl_xor_sync(full, m2, off);
+                        m2 = fminf(fmaxf(m1, o1), fminf(m2, o2));
+                        m1 = fminf(m1, o1);
+                    }
+                    s1 = slot_of_value(m1, -1);   // every lane takes part in the exchanges
+                }
                 const bool any = m1 < kInf;
-                int s1 = slot_of_value(m1, -1);   // every lane takes part in the exchanges
                 if (!any) s1 = 0;
                 const int tw = LA.t[s1], iw = any ? LA.idx[s1] : -2;
                 // C is in increasing scene index, hence in increasing time: the c with t'(c) <= x form a prefix, and
@@ -250,7 +333,12 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                 };
                 const int base_lane = lane & ~(TPB - 1);
                 int ccount, nT, pbs, pw;
-                {
+                if constexpr (kWarpRow) {
+                    ccount = inb ? entries_below<KM>(LC.t, nc, tb + 1, lane) : 0;
+                    nT = min(entries_below<KM>(LC.t, nc, T > 0 ? tw - T + 1 : INT32_MIN, lane), ccount);
+                    pbs = entry_at<KM>(LC.idx, nc, ib, lane);
+                    pw = entry_at<KM>(LC.idx, nc, iw, lane);
+                } else {
                     const int q = h & 3;
                     const int32_t *arr = q < 2 ? LC.t : LC.idx;
                     const int x = q == 0 ? tb + 1 : q == 1 ? (T > 0 ? tw - T + 1 : INT32_MIN) : q == 2 ? ib : iw;
@@ -273,13 +361,19 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     const bool has2 = m2 < kInf;
                     const int s2 = slot_of_value(m2, s1);
                     const int t2 = has2 ? LA.t[s2] : 0, i2 = has2 ? LA.idx[s2] : -2;
-                    const int q = h & 1;
-                    const int32_t *arr = q == 0 ? LC.t : LC.idx;
-                    const int x = q == 0 ? (T > 0 ? min(tw, t2) - T + 1 : INT32_MIN) : i2;
-                    int f = lower_bound(arr, x);
-                    if (q == 1 && !(f < nc && arr[f] == x)) f = KM;
-                    const int nT2 = min(__shfl_sync(full, f, base_lane), ccount);
-                    const int p2 = __shfl_sync(full, f, base_lane + 1);
+                    int nT2, p2;
+                    if constexpr (kWarpRow) {
+                        nT2 = min(entries_below<KM>(LC.t, nc, T > 0 ? min(tw, t2) - T + 1 : INT32_MIN, lane), ccount);
+                        p2 = entry_at<KM>(LC.idx, nc, i2, lane);
+                    } else {
+                        const int q = h & 1;
+                        const int32_t *arr = q == 0 ? LC.t : LC.idx;
+                        const int x = q == 0 ? (T > 0 ? min(tw, t2) - T + 1 : INT32_MIN) : i2;
+                        int f = lower_bound(arr, x);
+                        if (q == 1 && !(f < nc && arr[f] == x)) f = KM;
+                        nT2 = min(__shfl_sync(full, f, base_lane), ccount);
+                        p2 = __shfl_sync(full, f, base_lane + 1);
+                    }
                     // a c that rules out both: too far from both, or at one's point and too far from the other
                     loose = !has2 || nT2 - (pbs < nT2 ? 1 : 0) > 0 || p2 < nT || (pw < ccount && T > 0 && t2 - tw >= T);
                 }
@@ -293,11 +387,21 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     if (v[k] <= thr) mk |= 1u << k;
                 mk = ((mk << rot) | (mk >> (AH - rot))) & ((1u << AH) - 1);
                 int pos = 0, kept = __popc(mk);
+                if constexpr (kWarpRow) {
+                    kept = 0;
 #pragma unroll
-                for (int off = 1; off < TPB; off <<= 1) {
-                    const int o = __shfl_xor_sync(full, kept, off);
-                    if (h & off) pos += o;
-                    kept += o;
+                    for (int k = 0; k < AH; ++k) {
+                        const unsigned m = __ballot_sync(full, (mk >> k) & 1u);
+                        kept += __popc(m);
+                        pos += __popc(m & ((1u << lane) - 1));
+                    }
+                } else {
+#pragma unroll
+                    for (int off = 1; off < TPB; off <<= 1) {
+                        const int o = __shfl_xor_sync(full, kept, off);
+                        if (h & off) pos += o;
+                        kept += o;
+                    }
                 }
                 for (unsigned m = mk; m; m &= m - 1, ++pos) {
                     const int j = __ffs((int)m) - 1, a = AH * h + j;
@@ -323,8 +427,8 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // ---- phase 2: theta(a->c) for every a and the c = row with t'(c) <= t'(a). A kept a of a cell (b, c) has
             // t'(a) >= t'(b) >= t'(c), so only the rows from the first a with t'(a) >= t'(c) are read; entries of c
             // past the list belong to cells whose theta(b->c) is +inf, so their value is never used either
-            if (row < nc) {
-                const int c = row;
+            if (rowc < nc) {
+                const int c = rowc;
                 const int tc = LC.t[c], ic = LC.idx[c];
                 const float2 pc = LC.xy[c];
                 int lo = 0;
@@ -334,7 +438,7 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     else hi = mid;
                 }
 #pragma unroll 2
-                for (int a = lo + h; a < na; a += TPB) {
+                for (int a = lo + hc; a < na; a += TPC) {
                     const int ta = LA.t[a];
                     float r = direction(LA.xy[a], pc);   // theta(a->c)
                     if ((T > 0 && ta - tc >= T) || LA.idx[a] == ic) r = kInf;
@@ -346,20 +450,20 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // tile layout, by every thread (NT / KM per b): b's first tile = the tile count of the b ranked
             // before it (decreasing kept count, then increasing b)
             {
-                const int b = row, wb = sm.key(b), key = wb >> 5, nt_b = wb & 31;
+                const int b = rowc, wb = sm.key(b), key = wb >> 5, nt_b = wb & 31;
                 int before = 0, total = 0;
-                for (int b2 = h; b2 < KM; b2 += TPB) {
+                for (int b2 = hc; b2 < KM; b2 += TPC) {
                     const int w = sm.key(b2);
                     total += w & 31;
                     if ((w >> 5) > key) before += w & 31;
                 }
 #pragma unroll
-                for (int off = 1; off < TPB; off <<= 1) {
+                for (int off = 1; off < TPC; off <<= 1) {
                     before += __shfl_xor_sync(full, before, off);
                     total += __shfl_xor_sync(full, total, off);
                 }
-                if (h == 0) sm.info(b) = before << 12 | max((key >> 8) - 1, 0) << 5 | nt_b;
-                for (int t = h; t < nt_b; t += TPB) sm.tile_b(before + t) = (uint8_t)b;
+                if (hc == 0) sm.info(b) = before << 12 | max((key >> 8) - 1, 0) << 5 | nt_b;
+                for (int t = hc; t < nt_b; t += TPC) sm.tile_b(before + t) = (uint8_t)b;
                 if (tid == 0) {
                     sm.ntile = total;
                     sm.coin[(i - 1) & 1] = 0;
@@ -381,6 +485,14 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // ---- phase 3: tiles (b, CT consecutive c)
             const int ntile = sm.ntile;
             const bool coin = sm.coin[i & 1] != 0;
+            // where the next step's base of row c goes: the half of the CTA that owns the row
+            float *anext = sm.alpha + ((i - 1) & 1) * kHalf;
+            auto put = [&](int c, int b, float x) {
+                if constexpr (CL > 1)
+                    *cooperative_groups::this_cluster().map_shared_rank(anext + c * AS + b, (unsigned)c % CL) = x;
+                else
+                    sm.alpha[c * AS + b] = x;
+            };
             uint8_t *bstep = ubeta + (int64_t)(i - 2) * K * K;
             // tiles in decreasing kept count, dealt to the threads back and forth (round r: thread t takes
             // tile r NT + t for even r, r NT + NT - 1 - t for odd r) so that per-thread sums even out
@@ -459,7 +571,7 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
                     // alpha_i(b,c), and before the last step the next step's base: U(b) and the same Delta with it
                     const float al = cell_alpha(best[q], lam2, dt_bc, tb, tcq[q]);
                     const float out = i > 2 ? base_cost(ub, lam2, dt_bc, tb, tcq[q], al) : al;
-                    if (c < nc) sm.alpha[c * AS + b] = out;
+                    if (c < nc) put(c, b, out);
                     packed[q / 4] |= (uint32_t)arg[q] << (8 * (q % 4));
                 }
                 const bool aligned = (K & 3) == 0;
@@ -479,12 +591,13 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             // chain's cells are feasible) and the next step never reads their alpha (the pair (b, c) is
             // infeasible there); only the initial pair search of Eq. 13 reads every cell of the last step
             if (i == 2) {
-                for (int b = warp; b < nb; b += NW) {
+                for (int b = warp * CL + (int)rank; b < nb; b += NW * CL) {
                     const int covered = (sm.info(b) & 31) * CT;
-                    for (int c = covered + lane; c < nc; c += 32) sm.alpha[c * AS + b] = kInf;
+                    for (int c = covered + lane; c < nc; c += 32) put(c, b, kInf);
                 }
             }
-            __syncthreads();
+            if constexpr (CL > 1) cooperative_groups::this_cluster().sync();
+            else __syncthreads();
         }
 
         // Eq. 13: (z_1, z_2) = argmin U(z_1) + U(z_2) + alpha_3(z_2, z_1); ties -> lowest (z_1, z_2)
@@ -494,20 +607,30 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
             const int n0 = L0.n, n1 = L1.n;
             float bv = kInf;
             int bk = 0x7fffffff;
-            for (int e = tid; e < KM * KM; e += NT) {
-                const int c = e / KM, b = e % KM;    // e = z1 * KM + z2: lexicographic order
-                if (c < n0 && b < n1) argmin_merge(bv, bk, L0.u[c] + L1.u[b] + sm.alpha[c * AS + b], e);
+            const float *last = sm.alpha + kHalf;   // step 2 wrote the half of step 1
+            for (int e = tid; e < KM * KM / CL; e += NT) {
+                const int c = e / KM * CL + (int)rank, b = e % KM;    // z1 * KM + z2: lexicographic order
+                if (c < n0 && b < n1) argmin_merge(bv, bk, L0.u[c] + L1.u[b] + last[c * AS + b], CL > 1 ? c * KM + b : e);
             }
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1)
                 argmin_merge(bv, bk, __shfl_xor_sync(0xffffffffu, bv, off), __shfl_xor_sync(0xffffffffu, bk, off));
-            if (lane == 0) { sm.red_v[warp] = bv; sm.red_k[warp] = bk; }
-            __syncthreads();
-            if (warp == 0) {
+            if constexpr (CL > 1) {   // to CTA 0; the other CTAs' argmin bytes are visible to it after the barrier
+                if (lane == 0) {
+                    auto cl = cooperative_groups::this_cluster();
+                    *cl.map_shared_rank(&sm.red_v[rank * NW + warp], 0) = bv;
+                    *cl.map_shared_rank(&sm.red_k[rank * NW + warp], 0) = bk;
+                }
+                cooperative_groups::this_cluster().sync();
+            } else {
+                if (lane == 0) { sm.red_v[warp] = bv; sm.red_k[warp] = bk; }
+                __syncthreads();
+            }
+            if (warp == 0 && rank == 0) {
                 // every lane merges the warps' results: the same values
                 bv = sm.red_v[0];
                 bk = sm.red_k[0];
-                for (int w = 1; w < NW; ++w) argmin_merge(bv, bk, sm.red_v[w], sm.red_k[w]);
+                for (int w = 1; w < NW * CL; ++w) argmin_merge(bv, bk, sm.red_v[w], sm.red_k[w]);
                 const bool ok = bv < kInf;
                 const int z1 = ok ? bk / KM : -1, z2 = ok ? bk % KM : -1;
                 if constexpr (kFused)
@@ -519,6 +642,7 @@ recurse_kernel(const Unit *__restrict__ units, int64_t n_units, const ModelRec *
     }
 }
 
+constexpr int kURW = 4;      // unroll of the triple loop in the forms of one unit per SM or cluster
 constexpr int kFusedPerSm = 3;   // CTAs per SM of the fused variant (its argmin scratch is per CTA)
 
 struct FusedArgs {
@@ -529,18 +653,36 @@ struct FusedArgs {
     int32_t *assign = nullptr;
 };
 
-template <int KM, int NT, int MB, int CT, int UR, bool kCount, bool kFused>
+template <int KM, int NT, int MB, int CT, int UR, bool kCount, bool kFused, int CL = 1>
 cudaError_t launch_recurse_t(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
                              Params p, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
                              uint8_t *beta, UnitResult *res, int *work_counter, unsigned long long *evaluated,
                              const FusedArgs &fa, cudaStream_t st)
 {
     // three CTAs of 256 threads per SM: 3 x (shared memory + 1 KB reserved) <= 228 KB
-    static_assert(MB * (sizeof(Smem<KM, NT>) + 1024) <= 228 * 1024, "recursion shared memory exceeds the CTAs' budget");
-    auto kern = recurse_kernel<KM, NT, MB, CT, UR, kCount, kFused>;
-    const size_t smem = sizeof(Smem<KM, NT>);
+    static_assert(MB * (sizeof(Smem<KM, NT, CL>) + 1024) <= 228 * 1024, "recursion shared memory exceeds the CTAs' budget");
+    auto kern = recurse_kernel<KM, NT, MB, CT, UR, kCount, kFused, CL>;
+    const size_t smem = sizeof(Smem<KM, NT, CL>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    if constexpr (CL > 1) {   // a cluster per unit
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(n_units * CL));
+        cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CL;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        prof_begin(kProfRecurse, st);
+        e = cudaLaunchKernelEx(&cfg, kern, units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res,
+                               work_counter, evaluated, fa.n_dev, fa.n_from, fa.n_to, fa.beta_cta, fa.energy, fa.assign);
+        prof_end(kProfRecurse, st);
+        return e;
+    }
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -592,11 +734,34 @@ cudaError_t launch_wide(const Unit *units, int64_t n_units, const ModelRec *mode
                         UnitResult *res, int *work_counter, const FusedArgs &fa, cudaStream_t st)
 {
     if (p.K <= 32)
-        return launch_recurse_t<32, 256, 1, 4, 2, false, kFused>(units, n_units, models, scenes, p, cand_idx, cand_u,
+        return launch_recurse_t<32, 256, 1, 4, kURW, false, kFused>(units, n_units, models, scenes, p, cand_idx, cand_u,
                                                                  cand_cnt, beta, res, work_counter, nullptr, fa, st);
-    return launch_recurse_t<64, 512, 1, 4, 2, false, kFused>(units, n_units, models, scenes, p, cand_idx, cand_u,
+    return launch_recurse_t<64, 512, 1, 4, kURW, false, kFused>(units, n_units, models, scenes, p, cand_idx, cand_u,
                                                              cand_cnt, beta, res, work_counter, nullptr, fa, st);
 }
+
+// Few units: a cluster of four CTAs per unit, a warp per row in each, while the clusters of all units surely find
+// their SMs at once (five sixths of the SMs: clusters keep to one GPC). A step is then bound by its chain of
+// dependent operations: about 1,200 cycles (K = 32) and 2,200 (K = 64) of row lists, 1,400 and 2,300 of theta(a->c),
+// 2,000 and 4,000 of tiles, 1,000 of the cluster barrier. Two CTAs or half the threads per CTA were slower; theta(a->c)
+// computed by quarters and written to all four CTAs was too (its barrier costs more than the directions), and two or
+// four threads per tile changed nothing. 31 units of 16 points (K = 32): 67 -> 55 us; one to three fallback units of
+// 256 points (K = 64): 1,970 -> 1,430 us, both against one CTA per unit.
+constexpr int kCL = 4, kNT32 = 256, kNT64 = 512;
+
+template <bool kFused>
+cudaError_t launch_shared(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes, Params p,
+                          const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt, uint8_t *beta,
+                          UnitResult *res, int *work_counter, const FusedArgs &fa, cudaStream_t st)
+{
+    if (p.K <= 32)
+        return launch_recurse_t<32, kNT32, 1, 4, kURW, false, kFused, kCL>(units, n_units, models, scenes, p, cand_idx, cand_u,
+                                                                       cand_cnt, beta, res, work_counter, nullptr, fa, st);
+    return launch_recurse_t<64, kNT64, 1, 4, kURW, false, kFused, kCL>(units, n_units, models, scenes, p, cand_idx, cand_u,
+                                                                   cand_cnt, beta, res, work_counter, nullptr, fa, st);
+}
+
+int64_t shared_units(int64_t sms) { return sms * 5 / (6 * kCL); }
 
 int64_t wide_units()
 {
@@ -637,14 +802,16 @@ cudaError_t launch_model_geo(const float2 *xy, const int32_t *t, int M, float4 *
 cudaError_t preload_recurse()
 {
     cudaFuncAttributes a;
-    const void *kerns[] = {(const void *)recurse_kernel<32, 128, 4, 8, 2, false, false>,
-                           (const void *)recurse_kernel<32, 128, 4, 4, 4, false, false>,
-                           (const void *)recurse_kernel<32, 128, 4, 4, 2, false, false>,
-                           (const void *)recurse_kernel<64, 256, 3, 8, 2, false, false>,
-                           (const void *)recurse_kernel<64, 256, 3, 4, 4, false, false>,
-                           (const void *)recurse_kernel<64, 256, 3, 4, 2, false, false>,
-                           (const void *)recurse_kernel<32, 256, 1, 4, 2, false, false>,
-                           (const void *)recurse_kernel<64, 512, 1, 4, 2, false, false>};
+    const void *kerns[] = {(const void *)recurse_kernel<32, 128, 4, 8, 2, false, false, 1>,
+                           (const void *)recurse_kernel<32, 128, 4, 4, 4, false, false, 1>,
+                           (const void *)recurse_kernel<32, 128, 4, 4, 2, false, false, 1>,
+                           (const void *)recurse_kernel<64, 256, 3, 8, 2, false, false, 1>,
+                           (const void *)recurse_kernel<64, 256, 3, 4, 4, false, false, 1>,
+                           (const void *)recurse_kernel<64, 256, 3, 4, 2, false, false, 1>,
+                           (const void *)recurse_kernel<32, 256, 1, 4, kURW, false, false, 1>,
+                           (const void *)recurse_kernel<64, 512, 1, 4, kURW, false, false, 1>,
+                           (const void *)recurse_kernel<32, kNT32, 1, 4, kURW, false, false, kCL>,
+                           (const void *)recurse_kernel<64, kNT64, 1, 4, kURW, false, false, kCL>};
     for (const void *k : kerns) {
         cudaError_t e = cudaFuncGetAttributes(&a, k);
         if (e != cudaSuccess) return e;
@@ -661,9 +828,13 @@ cudaError_t launch_recurse(const Unit *units, int64_t n_units, const ModelRec *m
                            uint8_t *beta, UnitResult *res, int *work_counter, cudaStream_t st)
 {
     if (n_units <= 0) return cudaSuccess;
-    if (p.K <= 16)   // short lists (pruned form): one warp per unit
+    if (p.K <= 16)   // short lists (pruned form)
         return launch_recurse_small(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, st);
-    if (n_units <= wide_units())
+    const int64_t wide = wide_units();
+    if (n_units <= shared_units(wide))
+        return launch_shared<false>(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res,
+                                    work_counter, FusedArgs{}, st);
+    if (n_units <= wide)
         return launch_wide<false>(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, work_counter,
                                   FusedArgs{}, st);
     return dispatch<false, false>(g_variant, units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta,
@@ -691,13 +862,18 @@ cudaError_t launch_recurse_fused(const Unit *units, int64_t n_max, const int *n_
     fa.beta_cta = ((int64_t)std::max(max_M - 2, 1) * p.K * p.K + 255) / 256 * 256;
     fa.energy = energy;
     fa.assign = assign;
-    // the count is known on the device only: one launch for few units, one for more (an idle one costs 2-3 us)
-    const int few = (int)std::min<int64_t>(wide_units(), INT32_MAX);
-    fa.n_to = few;
-    cudaError_t e = launch_wide<true>(units, std::min<int64_t>(n_max, few), models, scenes, p, cand_idx, cand_u, cand_cnt,
-                                      scratch, nullptr, work_counter, fa, st);
+    // the count is known on the device only: a launch for every range of counts (an idle one costs 2-3 us)
+    const int64_t few = wide_units(), least = shared_units(few);
+    fa.n_to = (int)least;
+    cudaError_t e = launch_shared<true>(units, std::min(n_max, least), models, scenes, p, cand_idx, cand_u, cand_cnt,
+                                        scratch, nullptr, work_counter, fa, st);
+    if (e != cudaSuccess || n_max <= least) return e;
+    fa.n_from = (int)least;
+    fa.n_to = (int)few;
+    e = launch_wide<true>(units, std::min(n_max, few), models, scenes, p, cand_idx, cand_u, cand_cnt, scratch, nullptr,
+                          work_counter, fa, st);
     if (e != cudaSuccess || n_max <= few) return e;
-    fa.n_from = few;
+    fa.n_from = (int)few;
     fa.n_to = INT32_MAX;
     return dispatch<false, true>(0, units, n_max, models, scenes, p, cand_idx, cand_u, cand_cnt, scratch, nullptr,
                                  work_counter, nullptr, fa, st);

@@ -59,11 +59,33 @@ def test_few_and_many_units_give_the_same_bits(env, K):
     sc = _scene(rng, mod, 700, 12.0, 0.01)
     m, s = hgm.Model(mod.xy, mod.t, mod.f), hgm.Scene(sc.xy, sc.t, sc.f, sc.n_frames)
     first, e, a = hgm.match(m, s, hgm.default_params(K=K, window=3))
-    for lo, n in ((first, 1), (first + 100, 40), (first + 200, 160), (first + 5, 400)):
+    for lo, n in ((first, 1), (first + 300, 31), (first + 400, 32), (first + 100, 40), (first + 200, 160), (first + 5, 400)):
         p = hgm.default_params(K=K, window=3, offset_lo=lo, offset_hi=lo + n - 1)
         f1, e1, a1 = hgm.match(m, s, p)
         assert f1 == lo and len(e1) == n
         assert np.array_equal(e1, e[lo - first:lo - first + n]) and np.array_equal(a1, a[lo - first:lo - first + n])
+
+
+@pytest.mark.parametrize("K", [32, 64])
+@pytest.mark.parametrize("n", [1, 20, 100, 300])
+def test_fallback_of_few_and_many_units(env, K, n):
+    """A keep of one leaves a chain of this crowded scene without a feasible assignment almost everywhere: the
+    fallback's launches for few, some and many units give the exact path's bits on every unit they solve."""
+    torch, hgm, oracle = env
+    rng = np.random.default_rng(K)
+    mod = synth.make_model(rng, 14, F=16, frame=(60.0, 40.0), t_span=10)
+    sc = _scene(rng, mod, 700, 12.0, 0.01)
+    m, s = hgm.Model(mod.xy, mod.t, mod.f), hgm.Scene(sc.xy, sc.t, sc.f, sc.n_frames)
+    first, _ = hgm.offsets(m, s, hgm.default_params(K=K, window=3))
+    lo = first + 150
+    _, e, a = hgm.match(m, s, hgm.default_params(K=K, window=3, offset_lo=lo, offset_hi=lo + n - 1))
+    hgm.prune_counters(True)
+    prop = hgm.Proposal(16, seed=5)
+    p = hgm.default_params(K=K, window=3, prune=prop, keep=1, offset_lo=lo, offset_hi=lo + n - 1)
+    _, e1, a1 = hgm.match(m, s, p)
+    solved = e1 == e
+    assert solved.mean() > 0.9 and np.array_equal(a1[solved], a[solved])
+    assert np.all(e1[~solved] > e[~solved])
 
 
 @pytest.mark.parametrize("K,lam,crowd,T,window,M", [
