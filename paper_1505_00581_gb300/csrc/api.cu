@@ -204,10 +204,11 @@ struct hgm_stream {
     int32_t block_frames, F_user, Fp;
     int32_t max_points;                // capacity: points of one block (every buffer is sized for it at creation)
     hgm::BlockBufs bb;
-    hgm::Buffer sc_buf, raw;           // the block's sorted points (xy | t | perm | minnode), raw descriptors
+    // [energies | assignments] of host outputs, then what a block uploads in one copy: [flag (zero) | xy | t | perm |
+    // minnode | raw descriptors]. The flag is the descriptor check's, so the results and it are read back in one copy
+    hgm::Buffer sc_buf;
+    size_t o_assign = 0, o_flag = 0;   // offsets in sc_buf and in pin_out
     hgm::Buffer f;                     // sorted, padded descriptors
-    hgm::Buffer flag;
-    hgm::Buffer dev_e, dev_a;     // results before the read-back (host outputs)
     void *pin_out = nullptr;      // pinned read-back of energies, assignments and the flag
     size_t pin_out_bytes = 0;
     void *pinned = nullptr;       // host staging of the uploads
@@ -1887,10 +1888,11 @@ size_t al16(size_t v) { return (v + 15) & ~(size_t)15; }
 
 // Byte layout of a streamed block's upload: sorted xy | t | permutation | minnode table | raw descriptors.
 struct StreamUpload {
-    size_t o_t, o_perm, o_fs, o_raw;
+    size_t o_xy, o_t, o_perm, o_fs, o_raw;
     StreamUpload(int64_t n, int B)
     {
-        o_t = al16((size_t)n * 8);
+        o_xy = 16;   // after the flag
+        o_t = o_xy + al16((size_t)n * 8);
         o_perm = o_t + al16((size_t)n * 4);
         o_fs = o_perm + al16((size_t)n * 4);
         o_raw = o_fs + al16((size_t)(B + 1) * 4);
@@ -1914,13 +1916,11 @@ hgm_status stream_reserve(hgm_stream *s, int64_t P, cudaStream_t st)
     const size_t upload = up.o_raw + (size_t)P * F * sizeof(float);
     CK(cudaMallocHost(&s->pinned, upload), "pinned staging");
     s->pinned_bytes = upload;
-    CK(s->sc_buf.ensure(upload), "stream buffers");
+    s->o_assign = al16((size_t)nm * sizeof(float));
+    s->o_flag = s->o_assign + al16((size_t)R * sizeof(int32_t));
+    CK(s->sc_buf.ensure(s->o_flag + upload), "stream buffers");
     CK(s->f.ensure((size_t)std::max<int64_t>(P, 1) * Fp * sizeof(float)), "stream buffers");
-    CK(s->flag.ensure(sizeof(int)), "stream buffers");
-    CK(s->dev_e.ensure((size_t)nm * sizeof(float)), "stream buffers");
-    CK(s->dev_a.ensure((size_t)std::max<int64_t>(R, 1) * sizeof(int32_t)), "stream buffers");
-    const size_t o_a = al16((size_t)nm * sizeof(float));
-    s->pin_out_bytes = o_a + al16((size_t)R * sizeof(int32_t)) + 16;
+    s->pin_out_bytes = s->o_flag + 16;
     CK(cudaMallocHost(&s->pin_out, s->pin_out_bytes), "pinned staging");
     // run_block's buffers for one scene of P points
     BlockBufs &bb = s->bb;
@@ -2022,12 +2022,13 @@ hgm_status hgm_stream_match(hgm_stream *s, const float *xy, const int32_t *t, co
         for (int32_t k = 0; k < n; ++k) perm[(size_t)w[(size_t)ht[(size_t)k]]++] = k;
     }
     const StreamUpload up(n, B);
-    const size_t o_xy = 0, o_t = up.o_t, o_perm = up.o_perm, o_fs = up.o_fs, o_raw = up.o_raw;
+    const size_t o_xy = up.o_xy, o_t = up.o_t, o_perm = up.o_perm, o_fs = up.o_fs, o_raw = up.o_raw;
     const bool desc_dev = n > 0 && is_device_ptr(desc);
     const size_t total = o_raw + (desc_dev ? 0 : (size_t)n * F * sizeof(float));
     if (total > s->pinned_bytes) return fail(HGM_ECUDA, "stream staging smaller than its capacity (internal)");
     CK(cudaStreamSynchronize(st), "synchronise the staging buffer");   // the previous block's upload
     char *h = static_cast<char *>(s->pinned);
+    std::memset(h, 0, o_xy);
     float2 *sxy = reinterpret_cast<float2 *>(h + o_xy);
     int32_t *stt = reinterpret_cast<int32_t *>(h + o_t);
     for (int32_t k = 0; k < n; ++k) {
@@ -2038,17 +2039,13 @@ hgm_status hgm_stream_match(hgm_stream *s, const float *xy, const int32_t *t, co
     std::memcpy(h + o_perm, perm.data(), (size_t)n * 4);
     std::memcpy(h + o_fs, fs.data(), (size_t)(B + 1) * 4);
     if (!desc_dev && n > 0) std::memcpy(h + o_raw, desc, (size_t)n * F * sizeof(float));
-    CK(s->sc_buf.ensure(total), "stream buffers");
-    CK(s->f.ensure((size_t)std::max(n, 1) * Fp * sizeof(float)), "stream buffers");
-    CK(s->flag.ensure(sizeof(int)), "stream buffers");
-    CK(cudaMemcpyAsync(s->sc_buf.p, h, total, cudaMemcpyHostToDevice, st), "upload block");
-    char *d = s->sc_buf.as<char>();
-    CK(cudaMemsetAsync(s->flag.p, 0, sizeof(int), st), "memset");
+    char *dev = s->sc_buf.as<char>(), *d = dev + s->o_flag;
+    CK(cudaMemcpyAsync(d, h, total, cudaMemcpyHostToDevice, st), "upload block");
     if (n > 0) {
         const float *dsrc = desc_dev ? desc : reinterpret_cast<const float *>(d + o_raw);
         const int64_t blocks = std::min<int64_t>(((int64_t)n * Fp + 255) / 256, 65536);
         gather_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(dsrc, F, reinterpret_cast<const int32_t *>(d + o_perm), n,
-                                                             Fp, s->f.as<float>(), s->flag.as<int>());
+                                                             Fp, s->f.as<float>(), reinterpret_cast<int *>(d));
         CK(cudaGetLastError(), "gather kernel");
     }
     hgm_scene &v = s->view;
@@ -2065,28 +2062,24 @@ hgm_status hgm_stream_match(hgm_stream *s, const float *xy, const int32_t *t, co
     const size_t nm = ms.size();
     size_t a_total = 0;
     for (const hgm_model *m : ms) a_total += (size_t)m->d.M;
-    CK(s->dev_e.ensure(nm * sizeof(float)), "stream buffers");
-    CK(s->dev_a.ensure(std::max<size_t>(a_total, 1) * sizeof(int32_t)), "stream buffers");
-    rc = run_block(s->bb, ms.data(), (int)nm, &sv, 1, &s->params, st, s->dev_e.as<float>(), s->dev_a.as<int32_t>());
+    float *dev_e = reinterpret_cast<float *>(dev);
+    int32_t *dev_a = reinterpret_cast<int32_t *>(dev + s->o_assign);
+    rc = run_block(s->bb, ms.data(), (int)nm, &sv, 1, &s->params, st, dev_e, dev_a);
     if (rc) return rc;
-    const size_t o_a = al16(nm * sizeof(float));
-    const size_t o_f = o_a + al16(a_total * sizeof(int32_t));
-    if (o_f + 16 > s->pin_out_bytes) return fail(HGM_ECUDA, "stream read-back smaller than its capacity (internal)");
+    const size_t o_a = s->o_assign, o_f = s->o_flag;
     char *ho = static_cast<char *>(s->pin_out);
-    CK(cudaMemcpyAsync(ho, s->dev_e.p, nm * sizeof(float), cudaMemcpyDeviceToHost, st), "copy energy");
-    CK(cudaMemcpyAsync(ho + o_a, s->dev_a.p, a_total * sizeof(int32_t), cudaMemcpyDeviceToHost, st), "copy assign");
-    CK(cudaMemcpyAsync(ho + o_f, s->flag.p, sizeof(int), cudaMemcpyDeviceToHost, st), "flag");
+    CK(cudaMemcpyAsync(ho, dev, o_f + sizeof(int), cudaMemcpyDeviceToHost, st), "copy results");
     CK(cudaStreamSynchronize(st), "synchronise");
     int bad = 0;
     std::memcpy(&bad, ho + o_f, sizeof(int));
     if (bad) return fail(HGM_EINVAL, "non-finite block descriptor (outputs are not valid)");
     if (energy) {
         if (e_host) std::memcpy(energy, ho, nm * sizeof(float));
-        else CK(cudaMemcpyAsync(energy, s->dev_e.p, nm * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy energy");
+        else CK(cudaMemcpyAsync(energy, dev_e, nm * sizeof(float), cudaMemcpyDeviceToDevice, st), "copy energy");
     }
     if (assign) {
         if (a_host) std::memcpy(assign, ho + o_a, a_total * sizeof(int32_t));
-        else CK(cudaMemcpyAsync(assign, s->dev_a.p, a_total * sizeof(int32_t), cudaMemcpyDeviceToDevice, st),
+        else CK(cudaMemcpyAsync(assign, dev_a, a_total * sizeof(int32_t), cudaMemcpyDeviceToDevice, st),
                 "copy assign");
     }
     return HGM_OK;
