@@ -47,3 +47,12 @@ def test_block_many_pairs_equal_single_calls(env):  # noqa: F811
         e1, a1 = hgm.match_block([M[m]], [S[0]], p)
         assert e1[0] == e[2 * m]
         assert np.array_equal(a1, a[20 * m:20 * m + 10])
+
+
+@pytest.mark.parametrize("T", [0, 4500])
+def test_block_long_time_differences_take_the_general_form(env, T):  # noqa: F811
+    """Bands that span 4,096 frames or more do not fit a cell's record and take the kernel on global tables."""
+    torch, hgm, oracle = env
+    rng = np.random.default_rng(9)
+    mods = [synth.make_model(rng, M, F=16, frame=(60.0, 40.0), t_span=8) for M in (4, 7)]
+    _check(hgm, oracle, mods, [_uneven(rng, mods, 5000, 0.012, 0.05), _uneven(rng, mods, 4700, 0.006, 0.0)], T=T)
