@@ -42,9 +42,9 @@ L2_NOTE = "flushed (512 MiB write) before every step"
 # a small case, with the sources of the kernel it captured and the capture's argmin-table bytes
 # sum n_offsets (M - 2) K^2. Both the tables written and the lists read grow in proportion to that sum,
 # so a full launch's traffic is scaled by it; a changed kernel source voids the figure.
-RECURSE_NCU = {"sources_sha256": "015ced47a289cc2cc1d45f3754dcef8c424ddc24374815637abff006ea0717e5",
-               "bytes": 845_508_608 + 1_285_723_000, "beta_bytes": 1_667_760_128, "case": "combined_small"}
-RECURSE_SOURCES = ("k_recurse.cu", "recurse_common.cuh", "f32x2.cuh")
+RECURSE_NCU = {"sources_sha256": "334155295205910290c0fc7437be692215b119810b965463132898086b795981",
+               "bytes": 846_445_568 + 1_286_065_664, "beta_bytes": 1_667_760_128, "case": "combined_small"}
+RECURSE_SOURCES = ("k_recurse.cu", "recurse_common.cuh", "recurse_lists.cuh", "f32x2.cuh")
 
 
 def recurse_traffic(wl, chunks_per_step: int):
@@ -807,7 +807,7 @@ def main():
                          "frac": pairs_u * 2 * F_pad / (un_ms / 1e3) / 1e12 / peak_ops,
                          "work": f"{pairs_u:.4g} (model point, scene point) pairs x 2 x {F_pad} ops"},
         "select_kernel": {"bound": "latency", "lists_per_s": lists / (sel_ms / 1e3), "ms_per_step": sel_ms,
-                          "work": f"{lists} candidate lists (4 radix passes over each window)"}}
+                          "work": f"{lists} candidate lists (one or two rounds of bins over each window)"}}
     launches = sum(v[1] for v in prof.values())
 
     # the FP64 oracle on the host cores: all threads and one thread, on seeded units of this batch, which
