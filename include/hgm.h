@@ -231,7 +231,7 @@ HGM_API hgm_status hgm_match_block(const hgm_model *const *models, int32_t n_mod
  * blocks of about 60 frames, each matched whole against every model as it
  * arrives). A stream keeps the models' rows, the band and argmin tables and
  * pinned staging buffers between blocks, all sized at creation for blocks of
- * up to max_points points, so a block costs one upload, three kernel launches
+ * up to max_points points, so a block costs two uploads, three kernel launches
  * and the read-back of its results, and hgm_stream_match never allocates
  * device or pinned memory.
  * hgm_stream_create: models (handles; they must outlive the stream), params
@@ -319,8 +319,9 @@ HGM_API hgm_status hgm_prop_train_step(hgm_prop *prop, const float *X, const flo
 
 /* The recursion kernel (Eq. 10) comes in tile variants that differ only in how
  * the work is split (0: 4 z_{i-2} cells per thread, 1: 8 cells per thread,
- * 2: 4 cells per thread with half the threads per unit); results are
- * identical. hgm_autotune times every variant on this batch restricted to
+ * 2: 4 cells per thread, the triple loop unrolled further); results are
+ * identical. Caps K <= 16 and launches of at most one unit per SM take forms
+ * of their own, whatever the choice. hgm_autotune times every variant on this batch restricted to
  * offsets [max(offset_lo, 0), +sample_offsets) (full pipeline, CUDA events,
  * best of two after a warm-up), makes the fastest the process-wide choice and
  * returns it; ms_per_variant (host, may be NULL) receives each variant's time

@@ -2,10 +2,10 @@
 //
 // Same recursion as k_recurse.cu (Eqs. 10-13, readings R1-R6) for lists of at
 // most KS candidates. With K' = 8 a step has 64 cells of 8 candidates each, so
-// a whole CTA of the large-list kernel per unit would idle: here a group of warps (one for KS = 8, two or four for 16) owns a
-// unit, threads own cells (b, c) and minimise over a in slot order. Per step the per-(a, b) terms (base, p1,
-// p2) and the theta(a->c) table are computed once by the group; then a thread owns CT consecutive cells of one b. A
-// cell's result is written as the next step's base (as in k_recurse.cu), and the next step's list is fetched while
+// a whole CTA of the large-list kernel per unit would idle: here a group of warps (one for KS = 8, two or four for
+// 16) owns a unit, threads own cells (b, c) and minimise over a in slot order. Per step the per-(a, b) terms (base,
+// p1, p2) and the theta(a->c) table are computed once by the group; then a thread owns CT consecutive cells of one b.
+// A cell's result is written as the next step's base (as in k_recurse.cu), and the next step's list is fetched while
 // the tables are built. Every value is computed with the same FP32 operations in the same order as in the
 // large-list kernel (fast_atan2 directions, wrap, the two circular folds, sqrt.approx, fma; the model constants from
 // the same per-model table), so both kernels give the same bits.
