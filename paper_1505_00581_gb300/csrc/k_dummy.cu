@@ -357,8 +357,9 @@ __global__ void __launch_bounds__(NT, MB) dummy_recurse_kernel(
                 const float2 pb = LB.xy[b];
                 const int tb = LB.t[b], ib = LB.idx[b];
                 const float ub = LB.u[b], beb = sm.be(par, b);
-                // a real a of equal cost replaces eps: start just above base(eps, b)
-                const float start = __uint_as_float(__float_as_uint(beb) + 1u);
+                // a real a of equal cost replaces eps: start just above base(eps, b), but not above +inf (a dear
+                // dummy's sums overflow): the next bit pattern is a NaN, which no cost is below
+                const float start = beb < kInf ? __uint_as_float(__float_as_uint(beb) + 1u) : kInf;
                 float best[CT];
                 int arg[CT], tcq[CT];
                 bool open[CT];

@@ -37,3 +37,33 @@ def test_dummy_list_edges(K, lam, crowd, T, window, M, wd):
     for k in range(len(e)):
         ok, _, why = check_offset(orc, first + k, e[k], a[k])
         assert ok, (first + k, why)
+
+
+@pytest.mark.parametrize("K", [24, 64])
+@pytest.mark.parametrize("wd", [2e38, 1e38, 3e37, 1e37])
+def test_a_dummy_whose_sums_overflow_is_never_taken(K, wd):
+    """lambda1 W^d, or the sums of it along a chain, beyond FP32's largest value: eps costs +inf there, and every
+    offset that has a chain of real points keeps its plain optimum (of any W^d above, since one eps costs more)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1505_00581_gb300 import build, hgm
+    build.build()
+    import oracle
+    oracle.build()
+    rng = np.random.default_rng(0)
+    mod = synth.make_model(rng, 9, F=16, frame=(60.0, 40.0), t_span=10)
+    sc = synth.make_scene(rng, 30, (60.0, 40.0), ("poisson", 6.0), mod.centres, [mod], [(0, 2)])
+    m, s = hgm.Model(mod.xy, mod.t, mod.f), hgm.Scene(sc.xy, sc.t, sc.f, 30)
+    first, e, a = hgm.match(m, s, hgm.default_params(K=K, window=2, lambda1=2.0, dummy_cost=wd))
+    orc = oracle.Oracle(mod.xy, mod.t, mod.f, sc.xy, sc.t, sc.f, 30, K=K, window=2, T=10, lambda1=2.0, lambda2=0.2,
+                        lambda3=5.0)
+    feasible = 0
+    for k in range(len(e)):
+        if np.isfinite(orc.match(first + k)[0]):
+            ok, _, why = check_offset(orc, first + k, e[k], a[k])
+            assert ok, (first + k, why)
+            feasible += 1
+        elif 2.0 * wd > np.finfo(np.float32).max:
+            assert np.isinf(e[k]) and np.all(a[k] == -1)
+    assert feasible >= 10
