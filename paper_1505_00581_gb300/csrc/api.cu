@@ -605,7 +605,7 @@ hgm_status run_units(Exec &ex, const hgm_model *const *models, std::vector<Unit>
         }
         if (p.dummy >= 0) {
             // the dummy assignment: its own recursion kernel, which also backtracks
-            const int grid = dummy_grid(K);
+            const int grid = dummy_grid(K, max_M, (int64_t)std::max(budget, ws.beta_dummy.bytes));
             if (grid <= 0) return fail(HGM_ECUDA, "device query failed");
             CK(ws.beta_dummy.ensure((size_t)dummy_scratch_bytes(K, max_M, grid)), "workspace (argmin tables)");
             unsigned long long *ev = nullptr;

@@ -229,7 +229,7 @@ cudaError_t launch_block_recurse(const BlockUnit *units, int n_units, const Mode
 
 // k_dummy.cu: the recursion with the dummy assignment eps (fused backtrack; per-CTA argmin scratch).
 // evaluated != NULL runs the accounting variant, which adds its evaluated triples to *evaluated.
-int dummy_grid(int K);
+int dummy_grid(int K, int max_M, int64_t room);
 int64_t dummy_scratch_bytes(int K, int max_M, int grid);
 cudaError_t launch_recurse_dummy(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
                                  Params p, float wd, const int32_t *cand_idx, const float *cand_u,

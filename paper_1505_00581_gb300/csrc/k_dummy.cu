@@ -511,13 +511,17 @@ int64_t dummy_cta_bytes(int K, int max_M)
 
 int64_t dummy_scratch_bytes(int K, int max_M, int grid) { return grid * dummy_cta_bytes(K, max_M); }
 
-int dummy_grid(int K)
+// As many CTAs as fill the SMs, fewer where a long model's argmin scratch would take more than `room` bytes and more
+// than two CTAs per SM with tables of exactly (K+1)^2 would: 450,000 points at K = 4 are 535 MB per CTA, 325 GB in all.
+int dummy_grid(int K, int max_M, int64_t room)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                   cudaSuccess)
         return 0;
-    return sms * (K <= 32 ? kPerSm32 : kPerSm64);
+    const int64_t exact = (int64_t)sms * 2 * std::max(max_M - 2, 1) * (K + 1) * (K + 1);
+    const int64_t fit = std::max<int64_t>(std::max(room, exact) / dummy_cta_bytes(K, max_M), 1);
+    return (int)std::min<int64_t>(fit, sms * (K <= 32 ? kPerSm32 : kPerSm64));
 }
 
 cudaError_t launch_recurse_dummy(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,

@@ -1,5 +1,6 @@
 """The dummy-assignment recursion at the edges of its tables: caps around both table sizes and off the 4-cell tiles,
-crowded and empty windows, every closeness limit, a dummy that is free, cheap and dear, coincident points. Against
+crowded and empty windows, every closeness limit, a dummy that is free, cheap and dear (beyond FP32's range too),
+coincident points, a model whose tables would not fit a full grid. Against
 the FP64 oracle on every offset (energies 1e-5 relative, assignments equal or of the same FP64 energy)."""
 import numpy as np
 import pytest
@@ -67,3 +68,23 @@ def test_a_dummy_whose_sums_overflow_is_never_taken(K, wd):
         elif 2.0 * wd > np.finfo(np.float32).max:
             assert np.isinf(e[k]) and np.all(a[k] == -1)
     assert feasible >= 10
+
+
+def test_a_very_long_model_fits():
+    """450,000 model points at K = 4: the argmin tables of a full grid would take 325 GB. One far scene point, so that
+    every point takes eps: the energy is the sum of lambda1 W^d = 1/2, exact in FP32."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1505_00581_gb300 import build, hgm
+    build.build()
+    M = 450_000
+    m = hgm.Model(np.zeros((M, 2), np.float32), np.zeros(M, np.int32), np.zeros((M, 1), np.float32))
+    s = hgm.Scene(np.zeros((1, 2), np.float32), np.zeros(1, np.int32), np.full((1, 1), 8.0, np.float32), 1)
+    p = hgm.default_params(K=4, window=0, lambda1=0.5, dummy_cost=1.0, offset_lo=0, offset_hi=0)
+    hgm.set_workspace_budget(64 << 20)
+    try:
+        _, e, a = hgm.match(m, s, p)
+    finally:
+        hgm.set_workspace_budget(0)
+    assert e[0] == 0.5 * M and np.all(a == -2)
