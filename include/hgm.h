@@ -320,13 +320,17 @@ HGM_API hgm_status hgm_prop_train_step(hgm_prop *prop, const float *X, const flo
 /* The recursion kernel (Eq. 10) comes in tile variants that differ only in how
  * the work is split (0: 4 z_{i-2} cells per thread, 1: 8 cells per thread,
  * 2: 4 cells per thread, the triple loop unrolled further); results are
- * identical. Caps K <= 16 and launches of at most one unit per SM take forms
- * of their own, whatever the choice. hgm_autotune times every variant on this batch restricted to
+ * identical. Lists of at most 16 candidates, the dummy assignment and
+ * launches of at most one unit per SM take forms of their own, whatever the
+ * choice. hgm_autotune times every variant on this batch restricted to
  * offsets [max(offset_lo, 0), +sample_offsets) (full pipeline, CUDA events,
- * best of two after a warm-up), makes the fastest the process-wide choice and
- * returns it; ms_per_variant (host, may be NULL) receives each variant's time
- * (3 entries). hgm_set_recurse_variant restores
- * a cached choice. */
+ * best of two after a warm-up; the variant runs however few units that
+ * leaves), makes the fastest the process-wide choice and returns it;
+ * ms_per_variant (host, may be NULL) receives each variant's time (3
+ * entries). With lists of at most 16 (K, or keep with pruning) or the dummy
+ * assignment there is nothing to choose: the choice stays as it was and the
+ * three times are one measurement. hgm_set_recurse_variant restores a cached
+ * choice. */
 HGM_API hgm_status hgm_autotune(const hgm_model *const *models, int32_t n_models, const hgm_scene *const *scenes,
                                 int32_t n_scenes, const hgm_params *params, void *stream, int32_t sample_offsets,
                                 int32_t *best_variant, float *ms_per_variant);

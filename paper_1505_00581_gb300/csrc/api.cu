@@ -248,6 +248,7 @@ struct Exec {
     bool tensor = false;                                  // a tensor-core kernel ran (status flag is live)
     const std::vector<uint8_t> *select = nullptr;         // if set: only the units whose energy index is marked
     int64_t refined_units = 0;                            // units solved again by the refinement
+    bool tuning = false;                                  // the recursion's current variant, however few the units
 };
 
 hgm_status h2d(Exec &ex, void *dst, const void *src, size_t bytes, cudaStream_t st)
@@ -572,9 +573,9 @@ hgm_status run_units(Exec &ex, const hgm_model *const *models, std::vector<Unit>
             pk.K = keep;
             pk.rescore = 0;
             const Unit *du2 = ws.units2.as<Unit>();
-            CK(launch_recurse(du2, n, dm, ds, pk, ws.cand2_idx.as<int32_t>(), ws.cand2_u.as<float>(),
-                              ws.cand2_cnt.as<int32_t>(), ws.beta2.as<uint8_t>(), ws.res.as<UnitResult>(),
-                              ws.counter.as<int>(), st),
+            CK((ex.tuning ? launch_recurse_variant : launch_recurse)(
+                   du2, n, dm, ds, pk, ws.cand2_idx.as<int32_t>(), ws.cand2_u.as<float>(), ws.cand2_cnt.as<int32_t>(),
+                   ws.beta2.as<uint8_t>(), ws.res.as<UnitResult>(), ws.counter.as<int>(), st),
                "recursion kernel (pruned lists)");
             CK(launch_backtrack(du2, n, dm, ds, pk, ws.cand2_idx.as<int32_t>(), ws.beta2.as<uint8_t>(),
                                 ws.res.as<UnitResult>(), d_energy, d_assign, st),
@@ -627,9 +628,9 @@ hgm_status run_units(Exec &ex, const hgm_model *const *models, std::vector<Unit>
                                     ws.counter.as<int>(), ws.evaluated.as<unsigned long long>(), st),
                "recursion kernel (accounting)");
         } else {
-            CK(launch_recurse(du, n, dm, ds, p, ws.cand_idx.as<int32_t>(), ws.cand_u.as<float>(),
-                              ws.cand_cnt.as<int32_t>(), ws.beta.as<uint8_t>(), ws.res.as<UnitResult>(),
-                              ws.counter.as<int>(), st),
+            CK((ex.tuning ? launch_recurse_variant : launch_recurse)(
+                   du, n, dm, ds, p, ws.cand_idx.as<int32_t>(), ws.cand_u.as<float>(), ws.cand_cnt.as<int32_t>(),
+                   ws.beta.as<uint8_t>(), ws.res.as<UnitResult>(), ws.counter.as<int>(), st),
                "recursion kernel");
         }
         CK(launch_backtrack(du, n, dm, ds, p, ws.cand_idx.as<int32_t>(), ws.beta.as<uint8_t>(),
@@ -2304,17 +2305,24 @@ hgm_status hgm_autotune(const hgm_model *const *models, int32_t n_models, const 
     ps.offset_hi = (int32_t)std::min<int64_t>(params->offset_hi, (int64_t)ps.offset_lo + sample_offsets - 1);
     const int nv = recurse_variant_count();
     const int keep = get_recurse_variant();
+    // short lists and the dummy assignment have kernels of their own: nothing to choose
+    const bool choice = params->dummy_cost < 0 && (params->prune ? params->keep : params->K) > kShortK;
     cudaEvent_t a = nullptr, b = nullptr;
     CK(cudaEventCreate(&a), "event");
     CK(cudaEventCreate(&b), "event");
     float best_ms = 3.0e38f;
     int best = keep;
     for (int v = 0; v < nv; ++v) {
-        set_recurse_variant(v);
+        if (!choice && v > 0) {
+            if (ms_per_variant) ms_per_variant[v] = best_ms;
+            continue;
+        }
+        if (choice) set_recurse_variant(v);
         float vbest = 3.0e38f;
         for (int rep = 0; rep < 3; ++rep) {          // first repetition is a warm-up
             CK(cudaEventRecord(a, st), "event");
             Exec ex;
+            ex.tuning = choice;
             rc = run_batch(ex, models, n_models, scenes, n_scenes, &ps, st, nullptr, nullptr);
             if (rc) { set_recurse_variant(keep); cudaEventDestroy(a); cudaEventDestroy(b); return rc; }
             CK(cudaEventRecord(b, st), "event");
@@ -2324,7 +2332,7 @@ hgm_status hgm_autotune(const hgm_model *const *models, int32_t n_models, const 
             if (rep > 0) vbest = std::min(vbest, ms);
         }
         if (ms_per_variant) ms_per_variant[v] = vbest;
-        if (vbest < best_ms) { best_ms = vbest; best = v; }
+        if (vbest < best_ms) { best_ms = vbest; best = choice ? v : keep; }
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);

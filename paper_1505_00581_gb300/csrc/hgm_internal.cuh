@@ -146,7 +146,12 @@ cudaError_t launch_select(const Unit *units, int64_t n_units, const ModelRec *mo
 cudaError_t launch_recurse(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
                            Params p, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
                            uint8_t *beta, UnitResult *res, int *work_counter, cudaStream_t st);
-// k_recurse_small.cu: warp-per-unit recursion for lists of at most 16 candidates.
+// The current tile variant, however few the units (launch_recurse takes forms of its own for few units).
+cudaError_t launch_recurse_variant(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
+                                   Params p, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
+                                   uint8_t *beta, UnitResult *res, int *work_counter, cudaStream_t st);
+// k_recurse_small.cu: recursion for lists of at most kShortK candidates.
+constexpr int kShortK = 16;
 cudaError_t launch_recurse_small(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
                                  Params p, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
                                  uint8_t *beta, UnitResult *res, cudaStream_t st);

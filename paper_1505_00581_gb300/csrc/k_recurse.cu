@@ -828,7 +828,7 @@ cudaError_t launch_recurse(const Unit *units, int64_t n_units, const ModelRec *m
                            uint8_t *beta, UnitResult *res, int *work_counter, cudaStream_t st)
 {
     if (n_units <= 0) return cudaSuccess;
-    if (p.K <= 16)   // short lists (pruned form)
+    if (p.K <= kShortK)   // short lists (pruned form)
         return launch_recurse_small(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, st);
     const int64_t wide = wide_units();
     if (n_units <= shared_units(wide))
@@ -837,6 +837,14 @@ cudaError_t launch_recurse(const Unit *units, int64_t n_units, const ModelRec *m
     if (n_units <= wide)
         return launch_wide<false>(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, work_counter,
                                   FusedArgs{}, st);
+    return launch_recurse_variant(units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta, res, work_counter, st);
+}
+
+cudaError_t launch_recurse_variant(const Unit *units, int64_t n_units, const ModelRec *models, const SceneRec *scenes,
+                                   Params p, const int32_t *cand_idx, const float *cand_u, const int32_t *cand_cnt,
+                                   uint8_t *beta, UnitResult *res, int *work_counter, cudaStream_t st)
+{
+    if (n_units <= 0) return cudaSuccess;
     return dispatch<false, false>(g_variant, units, n_units, models, scenes, p, cand_idx, cand_u, cand_cnt, beta,
                                   res, work_counter, nullptr, FusedArgs{}, st);
 }

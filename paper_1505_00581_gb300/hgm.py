@@ -8,6 +8,7 @@ CUDA stream, and raises on a non-zero status. There is no CPU fallback: if
 from __future__ import annotations
 
 import ctypes
+import hashlib
 import os
 from typing import Sequence
 
@@ -354,13 +355,17 @@ def _tune_key(params: Params) -> str:
         dev = torch.cuda.get_device_name() if torch.cuda.is_available() else "none"
     except ImportError:
         dev = "unknown"
-    return f"{dev}|K{'<=32' if params.K <= 32 else '<=64'}|precision{params.precision}"
+    with open(LIB_PATH, "rb") as fh:      # a choice among kernels that were built anew since says nothing
+        lib = hashlib.sha256(fh.read()).hexdigest()[:12]
+    return f"{dev}|K{'<=32' if params.K <= 32 else '<=64'}|precision{params.precision}|lib {lib}"
 
 
 def autotune(models: Sequence[Model], scenes: Sequence[Scene], params: Params, sample_offsets: int = 128,
              use_cache: bool = True, stream=None):
     """Picks the fastest recursion tile variant for this workload (hgm_autotune) and caches the choice
-    in a JSON file keyed by device name and K bucket. Returns (variant, {variant: ms} or None)."""
+    in a JSON file keyed by device name, K bucket, precision and the library's build. Returns (variant,
+    {variant: ms} or None). Where there is nothing to choose (hgm_autotune says when: three equal times), the
+    current variant stays and nothing is cached."""
     import json
     lib = load()
     key, path = _tune_key(params), _tune_cache_path()
@@ -381,7 +386,7 @@ def autotune(models: Sequence[Model], scenes: Sequence[Scene], params: Params, s
     _check(lib.hgm_autotune(mh, nm, sh, ns, ctypes.byref(params), _stream(stream), int(sample_offsets),
                             ctypes.byref(best), ms.ctypes.data_as(_pf)))
     times = {v: float(ms[v]) for v in range(N_VARIANTS)}
-    if use_cache:
+    if use_cache and len(set(times.values())) > 1:
         cache[key] = {"variant": int(best.value), "ms": times, "sample_offsets": int(sample_offsets)}
         try:
             os.makedirs(os.path.dirname(path), exist_ok=True)

@@ -88,6 +88,38 @@ def test_fallback_of_few_and_many_units(env, K, n):
     assert np.all(e1[~solved] > e[~solved])
 
 
+def test_autotune_times_the_variants_on_a_small_sample(env):
+    """One unit takes a cluster of four CTAs in a call, a variant's single CTA in the tuner: about twice as long
+    for the 126 steps here. Tuning that ran the call's own form would show the same time."""
+    torch, hgm, oracle = env
+    rng = np.random.default_rng(4)
+    mod = synth.make_model(rng, 128, F=16, frame=(60.0, 40.0), t_span=30)
+    m = hgm.Model(mod.xy, mod.t, mod.f)
+    sc = _scene(rng, mod, 60, 12.0, 0.0)
+    s = hgm.Scene(sc.xy, sc.t, sc.f, sc.n_frames)
+    p = hgm.default_params(K=64, window=3, offset_lo=5, offset_hi=5)
+
+    def ms_per_launch(fn):
+        hgm.profile_reset()
+        hgm.profile_enable(True)
+        fn()
+        hgm.profile_enable(False)
+        ms, n = hgm.profile_read()["recurse"]
+        return ms / n
+
+    hgm.set_recurse_variant(0)
+    hgm.match(m, s, p)
+    call = min(ms_per_launch(lambda: hgm.match(m, s, p)) for _ in range(5))
+    tuned = ms_per_launch(lambda: hgm.autotune([m], [s], p, use_cache=False))
+    assert tuned > 1.4 * call, (tuned, call)
+    # nothing to choose: the choice stays, the three times are one measurement
+    hgm.set_recurse_variant(2)
+    for kw in (dict(K=16), dict(K=64, dummy_cost=4.0)):
+        best, ms = hgm.autotune([m], [s], hgm.default_params(window=3, offset_lo=5, offset_hi=5, **kw), use_cache=False)
+        assert best == 2 and len(set(ms.values())) == 1
+    hgm.set_recurse_variant(0)
+
+
 @pytest.mark.parametrize("K,lam,crowd,T,window,M", [
     (1, 3.0, 0.0, 10, 1, 5), (5, 6.0, 0.2, 10, 2, 9), (8, 20.0, 0.0, 4, 2, 8), (9, 8.0, 0.1, 10, 2, 10),
     (13, 20.0, 0.3, 0, 2, 7), (16, 30.0, 0.0, 10, 1, 3), (16, 1.0, 0.2, 10, 3, 20), (15, 12.0, 0.0, 2, 3, 9)])
