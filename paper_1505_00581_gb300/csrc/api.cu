@@ -1981,7 +1981,12 @@ hgm_status hgm_stream_create(const hgm_model *const *models, int32_t n_models, c
     cudaStream_t st = (cudaStream_t)stream;
     rc = prep_block_models(s->bb, s->models.data(), n_models, st);
     if (!rc) rc = stream_reserve(s, max_points, st);
-    cudaError_t e = cudaStreamSynchronize(st);
+    // the kernels of a block of any shape: their code is loaded now as well
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, gather_rows_kernel);
+    if (e == cudaSuccess) e = preload_unary();
+    if (e == cudaSuccess) e = preload_block();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (!rc && e != cudaSuccess) rc = cuda_fail(e, "stream create");
     if (rc) {
         free_stream(s);

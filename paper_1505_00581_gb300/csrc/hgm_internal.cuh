@@ -187,6 +187,7 @@ cudaError_t preload_select();
 cudaError_t preload_recurse();
 cudaError_t preload_recurse_small();
 cudaError_t preload_backtrack();
+cudaError_t preload_block();
 
 // Profiling hooks (api.cu).
 // k_block.cu: the whole-block problem (every scene point a candidate, no offsets).

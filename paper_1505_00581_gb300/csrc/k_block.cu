@@ -613,6 +613,29 @@ BlockPlan block_plan(const BlockBand *bands, int n_scenes, int n_units, int max_
     return pl;
 }
 
+cudaError_t preload_block()
+{
+    cudaFuncAttributes a;
+    const void *kerns[] = {(const void *)block_cluster_kernel<256, false, false>,
+                           (const void *)block_cluster_kernel<256, false, true>,
+                           (const void *)block_cluster_kernel<256, true, false>,
+                           (const void *)block_cluster_kernel<512, false, false>,
+                           (const void *)block_cluster_kernel<512, false, true>,
+                           (const void *)block_cluster_kernel<512, true, false>,
+                           (const void *)block_cluster_kernel<1024, false, false>,
+                           (const void *)block_cluster_kernel<1024, false, true>,
+                           (const void *)block_cluster_kernel<1024, true, false>,
+                           (const void *)block_recurse_kernel<kBlockThreads>,
+                           (const void *)block_recurse_kernel<kBlockThreadsWide>,
+                           (const void *)block_cells_kernel,
+                           (const void *)block_dirs_kernel};
+    for (const void *k : kerns) {
+        cudaError_t e = cudaFuncGetAttributes(&a, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 bool block_always_shared(int64_t points, int n_frames, int T)
 {
     if ((T > 0 ? std::min(T, n_frames) : n_frames) > 1 << 12) return false;
