@@ -496,11 +496,13 @@ cudaError_t PropTrain::ensure(const PropLayout &L, int B)
     buf = nullptr;
     cap = 0;
     const size_t shares = (size_t)pass_ctas(L, B) * (size_t)L.n;
-    cudaError_t e = cudaMalloc(&buf, (shares + 8) * sizeof(float));
+    const size_t logits = ((size_t)B + 3) & ~(size_t)3;
+    cudaError_t e = cudaMalloc(&buf, (shares + logits + 8) * sizeof(float));
     if (e != cudaSuccess) return e;
     float *q = static_cast<float *>(buf);
     part = q;                  // L.n is a multiple of 4: the words after stay aligned
-    loss = q + shares;
+    z3 = q + shares;
+    loss = z3 + logits;
     status = reinterpret_cast<int *>(loss + 4);
     cap = B;
     return cudaMemset(status, 0, sizeof(int));

@@ -21,6 +21,7 @@ struct PropTrain {
     void *buf = nullptr;
     int cap = 0;
     float *part = nullptr;   // per CTA of a pass: its share of the gradient, L.n floats
+    float *z3 = nullptr;     // logits of a forward pass whose output lies in its input
     float *loss = nullptr;   // mean loss of the last pass
     int *status = nullptr;   // 1 once a bounded tensor-core wait gave up
     cudaError_t ensure(const PropLayout &L, int B);

@@ -116,8 +116,14 @@ hgm_status hgm_prop_forward(hgm_prop *prop, const float *X, int32_t B, void *str
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = prop->train.ensure(prop->L, B))) return cuerr(e, "workspace");
-    if ((e = prop_forward(prop->L, prop->theta, prop->train, X, prop->L.d_in, B, logits, st)))
+    // the pass writes a tile's logits while others' rows are still read: where they lie in X, they wait in the workspace
+    const uintptr_t x = (uintptr_t)X, z = (uintptr_t)logits;
+    const bool inside = z < x + sizeof(float) * (size_t)B * prop->L.d_in && x < z + sizeof(float) * (size_t)B;
+    float *out = inside ? prop->train.z3 : logits;
+    if ((e = prop_forward(prop->L, prop->theta, prop->train, X, prop->L.d_in, B, out, st)))
         return cuerr(e, "forward");
+    if (inside && (e = cudaMemcpyAsync(logits, out, sizeof(float) * B, cudaMemcpyDeviceToDevice, st)))
+        return cuerr(e, "copy");
     return check_status(prop, st);
 }
 

@@ -97,3 +97,18 @@ def test_step_equals_gradients_and_adam(env):
         want = w - 1e-3 * (m / (1 - 0.9 ** t)) / (np.sqrt(v / (1 - 0.999 ** t)) + 1e-8)
         # FP32: c2 = 1 - 0.999^t keeps 2^-24 / 0.001 = 6e-5 of relative error, the update half of that
         assert np.max(np.abs(prop.get()[0] - want)) <= 1e-3 * 1e-4 + 2.0 ** -23 * np.max(np.abs(w))
+
+
+@pytest.mark.parametrize("at", [0, 7, -1])
+def test_logits_may_lie_in_the_input(env, at):
+    """313 tiles on 152 SMs: the first round's logits would land in rows that the later rounds still read."""
+    torch, hgm = env
+    B, F = 40000, 1
+    prop = hgm.Proposal(F, seed=9)
+    X = torch.from_numpy(np.random.default_rng(9).normal(size=(B, 2 * F + 3)).astype(np.float32)).cuda()
+    want = torch.empty(B, device="cuda")
+    prop.forward(X, want)
+    flat = X.view(-1)
+    out = flat[flat.numel() - B:] if at < 0 else flat[at:at + B]
+    prop.forward(X, out)
+    assert torch.equal(out, want)
