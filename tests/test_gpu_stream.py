@@ -166,15 +166,18 @@ _FIRST_BLOCK = """
 import sys, time
 sys.path[:0] = [{root!r}]
 import numpy as np
+import torch
 from paper_1505_00581_gb300 import hgm, synth
 r = np.random.default_rng(0)
 mods = [synth.make_model(r, 12, F=32, frame=(160.0, 120.0), t_span=12) for _ in range(3)]
 M = [hgm.Model(x.xy, x.t, x.f) for x in mods]
-st = hgm.Stream(M, hgm.default_params(T=10), 60, max_points=200)
-t = np.sort(r.integers(0, 60, 20)).astype(np.int32)
-xy, f = r.random((20, 2)).astype(np.float32), r.normal(size=(20, 32)).astype(np.float32)
+torch.cuda.synchronize()
+st = hgm.Stream(M, hgm.default_params(T=10), 60, max_points=800)
+torch.cuda.synchronize()
 us = []
 for _ in range(12):
+    t = np.sort(r.integers(0, 60, 20)).astype(np.int32)
+    xy, f = r.random((20, 2)).astype(np.float32), r.normal(size=(20, 32)).astype(np.float32)
     a = time.perf_counter()
     st.match(xy, t, f)
     us.append(time.perf_counter() - a)
@@ -184,8 +187,8 @@ print(us[0] / np.median(us[2:]))
 
 def test_first_block_loads_no_kernels(env):
     """hgm_stream_match allocates no device memory, so the code of every kernel a block can take is loaded when the
-    stream is created. In a process of its own, the first block took 4.3 to 4.5 times as long as later ones with the
-    kernels loaded on the way, and takes 1.4 to 1.6 times as long without (the best of three runs counts)."""
+    stream is created. In a process of its own, the first block took 5.4 to 6.1 times as long as later ones with the
+    kernels loaded on the way, and takes 1.9 to 2.4 times as long without (the best of three runs counts)."""
     import os
     import subprocess
     import sys
@@ -195,6 +198,6 @@ def test_first_block_loads_no_kernels(env):
         r = subprocess.run([sys.executable, "-c", _FIRST_BLOCK.format(root=root)], capture_output=True, text=True, timeout=300)
         assert r.returncode == 0, r.stderr
         ratios.append(float(r.stdout.split()[-1]))
-        if ratios[-1] < 2.5:
+        if ratios[-1] < 3.5:
             return
-    assert min(ratios) < 2.5, ratios
+    assert min(ratios) < 3.5, ratios
