@@ -1901,8 +1901,9 @@ struct StreamUpload {
 };
 
 // Every buffer a block of up to P points can need, allocated once: the upload staging (pinned) and its device
-// copy, the sorted descriptors, the band tables (at most P cells per point: a band holds points of the block),
-// the unary and argmin tables, the global alpha scratch when a band exceeds shared memory, the outputs.
+// copy, the sorted descriptors, the band starts (at most P cells per point: a band holds points of the block),
+// the unary and argmin tables, the general form's band tables and alpha scratch when a band may exceed shared
+// memory, the outputs.
 hgm_status stream_reserve(hgm_stream *s, int64_t P, cudaStream_t st)
 {
     (void)st;
@@ -1932,13 +1933,13 @@ hgm_status stream_reserve(hgm_stream *s, int64_t P, cudaStream_t st)
     CK(bb.tab.ensure(tab), "stream buffers");
     CK(cudaMallocHost(&bb.pinned, tab), "pinned staging");
     bb.pinned_bytes = tab;
-    CK(bb.cellb.ensure((size_t)cells * sizeof(int32_t)), "stream buffers");
-    CK(bb.dir.ensure((size_t)cells * 2 * sizeof(float)), "stream buffers");
     CK(bb.U.ensure((size_t)std::max<int64_t>(P * R, 1) * sizeof(float)), "stream buffers");
     CK(bb.beta.ensure((size_t)std::max<int64_t>(Rm2 * cells, 1) * sizeof(uint16_t)), "stream buffers");
     CK(bb.oe.ensure((size_t)nm * sizeof(float)), "stream buffers");
     CK(bb.oa.ensure((size_t)std::max<int64_t>(R, 1) * sizeof(int32_t)), "stream buffers");
-    if (!block_always_shared(P, B, s->params.T)) {
+    if (!block_always_shared(P, B, s->params.T)) {   // some block may take the general form
+        CK(bb.cellb.ensure((size_t)cells * sizeof(int32_t)), "stream buffers");
+        CK(bb.dir.ensure((size_t)cells * 2 * sizeof(float)), "stream buffers");
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev), "device");
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device");

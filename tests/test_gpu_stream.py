@@ -201,3 +201,25 @@ def test_first_block_loads_no_kernels(env):
         if ratios[-1] < 3.5:
             return
     assert min(ratios) < 3.5, ratios
+
+
+@pytest.mark.parametrize("cap", [86, 87])
+def test_capacities_around_the_shared_memory_limit(env, cap):
+    """Up to 86 points every block fits one CTA's shared memory and the stream keeps no tables of the general form;
+    87 is the first that keeps them. Blocks at the capacity, all points in one frame (the largest band), in two, and
+    spread: the same bits as hgm_match_block."""
+    torch, hgm, oracle = env
+    mods, _ = _long_scene(9, n_models=2)
+    M = [hgm.Model(m.xy, m.t, m.f) for m in mods]
+    p = hgm.default_params()
+    st = hgm.Stream(M, p, 60, max_points=cap)
+    rng = np.random.default_rng(cap)
+    xy = (rng.random((cap, 2)) * (160.0, 120.0)).astype(np.float32)
+    f = rng.normal(size=(cap, mods[0].F)).astype(np.float32)
+    for t in (np.full(cap, 30), 20 + np.arange(cap) % 2, np.sort(rng.integers(0, 60, cap))):
+        t = t.astype(np.int32)
+        e, a = st.match(xy, t, f)
+        e2, a2 = hgm.match_block(M, [hgm.Scene(xy, t, f, 60)], p)
+        np.testing.assert_array_equal(e, e2)
+        np.testing.assert_array_equal(a, a2)
+    st.close()
