@@ -1,6 +1,6 @@
 """The recursion kernel at the edges of its lists: caps around the two table sizes and off the 4-cell tiles, lists
 shorter than the cap and of very different lengths, crowded frames (many points of equal time), every closeness
-limit, points shared between lists, small and large numbers of units. Against the FP64 oracle on every offset
+limit, points shared between lists, numbers of units for every form of the launch. Against the FP64 oracle on every offset
 (tests/gpu_util.check_offset: energies 1e-5 relative, assignments equal or of the same FP64 energy)."""
 import numpy as np
 import pytest
@@ -48,6 +48,16 @@ def test_list_edges(env, K, lam, crowd, T, window, M):
     for k in range(len(e)):
         ok, _, why = check_offset(orc, first + k, e[k], a[k])
         assert ok, (first + k, why)
+    # the same pair several times over: enough units for each form of the launch (a cluster per unit, a unit per SM,
+    # the variants; with short lists four warps per unit, then two), whose bits must be those of the one pair
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for units in (sms // 2, 9 * sms):
+        n = -(-units // len(e))
+        eb = np.empty(n * e.size, np.float32)
+        ab = np.empty(n * a.size, np.int32)
+        hgm.match_batch([m] * n, [s], p, eb, ab)
+        assert np.array_equal(eb.reshape(n, -1), np.broadcast_to(e, (n, e.size)))
+        assert np.array_equal(ab.reshape(n, -1), np.broadcast_to(a.reshape(-1), (n, a.size)))
 
 
 @pytest.mark.parametrize("K", [32, 64])
