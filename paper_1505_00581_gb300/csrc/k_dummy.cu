@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(NT, MB) dummy_recurse_kernel(
                 const float ub = LB.u[b], beb = sm.be(par, b);
                 // a real a of equal cost replaces eps: start just above base(eps, b), but not above +inf (a dear
                 // dummy's sums overflow): the next bit pattern is a NaN, which no cost is below
-                const float start = beb < kInf ? __uint_as_float(__float_as_uint(beb) + 1u) : kInf;
+                const float start = __uint_as_float(min(__float_as_uint(beb) + 1u, __float_as_uint(kInf)));
                 float best[CT];
                 int arg[CT], tcq[CT];
                 bool open[CT];

@@ -12,8 +12,8 @@
 namespace hgm {
 
 // Approximate square root of a squared angle difference. Flushing subnormal inputs (angle differences below
-// 1.1e-19) saves the compiler's rescaling around the instruction, three more per triple; such a difference is
-// far below an ulp of any angle it is added to.
+// 1.1e-19) saves the compiler's rescaling around the instruction, three more per triple. It moves a triple's cost by
+// at most lambda2 lambda3 1.1e-19; the FP32 directions the difference is formed from are off by up to 6e-7.
 __device__ __forceinline__ float sqrt_fast(float x)
 {
     float r;
