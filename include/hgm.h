@@ -231,9 +231,10 @@ HGM_API hgm_status hgm_match_block(const hgm_model *const *models, int32_t n_mod
  * blocks of about 60 frames, each matched whole against every model as it
  * arrives). A stream keeps the models' rows, the band and argmin tables and
  * pinned staging buffers between blocks, all sized at creation for blocks of
- * up to max_points points, so a block costs two uploads, three kernel launches
- * and the read-back of its results, and hgm_stream_match never allocates
- * device or pinned memory.
+ * up to max_points points, and the kernels' code is loaded there, so a block
+ * costs two uploads, three kernel launches (five where its band fits no
+ * cluster's shared memory or spans 4,096 frames) and the read-back of its
+ * results, and hgm_stream_match never allocates device or pinned memory.
  * hgm_stream_create: models (handles; they must outlive the stream), params
  * as for hgm_match_block, block_frames >= 1 (frames of one block),
  * max_points >= 1 (the largest block; the band tables are sized for

@@ -183,9 +183,10 @@ __global__ void __launch_bounds__(NT, 1) block_recurse_kernel(
 //
 // Bound by shared memory: per two a of 32 cells three 8-byte and two 4-byte loads of rows that lie apart (about 15
 // wavefronts for 43 instructions; two thirds of the cycles on Table 2's scene). Measured with the earlier kernel
-// (tables in global memory, five dependent gathers per a, one CTA per pair) and with this one: 50 pairs of 11,700
-// cells 2,325 -> 434 us (two CTAs per pair; 46 clusters of three fit the chip, not 50), 50 pairs of 1,800 cells
-// (a 60-frame block) 325 -> 90 us. Ordering the cells took 31% of the instructions and 2% of the time.
+// (tables in global memory, five dependent gathers per a, one CTA per pair) and with this one, by CUDA events: 50
+// pairs of 10,000 cells (788 points over 723 frames) 1,653 -> 258 us (two CTAs per pair; 46 clusters of three fit the
+// chip, not 50), 50 pairs of 1,270 cells (86 points over 60 frames) 282 -> 100 us. Ordering the cells took 31% of the
+// instructions and 2% of the time.
 struct BlockPt {
     float2 xy;
     int t, flo, fhi, fr, lo, cs;   // fr: first entry of the point's row, cs: its first cell (whole scene)

@@ -14,8 +14,8 @@
 //  * the cells that hold eps are minima without a geometric term: (b, eps) over the a within T of b, by the row's
 //    threads; (eps, c) over base(a, eps), by the threads of c; (eps, eps) by one warp. Their base values are three
 //    small arrays, kept for the coming and the current step.
-// Ties prefer the lower slot, eps last: a cell's walk starts from the next float above base(eps, b), so a real a of
-// equal cost replaces it. The argmin slots go to a per-CTA global scratch, and the CTA backtracks its own unit (Eq.
+// Ties prefer the lower slot, eps last: a cell's walk starts from the next float above base(eps, b), at most +inf, so a
+// real a of equal cost replaces it. The argmin slots go to a per-CTA global scratch, and the CTA backtracks its own unit (Eq.
 // 12); eps is reported as -2 in the assignment.
 //
 // Bound by issue and the latency of the step's phases. Measured with the earlier kernel (a warp per row ranking the

@@ -124,7 +124,8 @@ __device__ __forceinline__ float column_sum(float (&v)[32], int lane)
 // F = 162: 2.28 ms per step with one kernel per operation (the weight gradients were one-CTA products over the
 // whole batch, 1.1 ms each, the column sums one-CTA loops, 0.4 ms each), 0.06 ms with this pass, weight transfer
 // included. 128 rows per tile because that is the product's M; four warps per 32 rows because a warp reads only
-// its quarter of tensor memory and 32 columns leave the epilogue in registers.
+// its quarter of tensor memory and 32 columns leave the epilogue in registers (all but 13 words of the 128 registers
+// that 512 threads have).
 template <bool kTrain>
 __global__ void __launch_bounds__(NT, 1) prop_pass_kernel(PropLayout L, const float *__restrict__ theta,
                                                           const float *__restrict__ X, int64_t ldx,

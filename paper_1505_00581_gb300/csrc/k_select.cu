@@ -39,7 +39,7 @@ static_assert(32 % kRescoreMax == 0, "whole lists fill a warp");
 // kKeyRegs keys per lane are held in registers: windows of up to 32 kKeyRegs keys are selected from them,
 // longer ones from memory in every pass. The launch picks 8 (three CTAs per SM) when the call's typical
 // window (the scenes' mean density over 2w+1 frames) fits 256 keys, else 20 (two CTAs per SM, the registers
-// the larger arrays need).
+// the larger arrays need). At the 80 registers that three CTAs leave, seven words of the first are spilled.
 template <int kKeyRegs, int kMinBlocks>
 __global__ void __launch_bounds__(kWarps * 32, kMinBlocks) select_kernel(const Unit *__restrict__ units, int64_t n_units,
                                                              const ModelRec *__restrict__ models,
